@@ -92,7 +92,7 @@ typedef struct wrs_table wrs_table; /* opaque; device memory owned by the librar
  * rebuilt any number of times.  Every later call on a table records CUDA
  * events on the streams it is given, so that the host-side calls below wait
  * for this table's work only.  Device memory: 16 B per bucket plus about
- * 0.09 B per weight of workspace.  Errors: WRS_EINVAL, WRS_ENOMEM. */
+ * 0.1 B per weight of workspace (0.65 B for each of the first 2^22).  Errors: WRS_EINVAL, WRS_ENOMEM. */
 wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out);
 
 /* Build the alias table of n weights (Alg. 3 "PSA", Sec. 4.2, with the exact
@@ -107,13 +107,13 @@ wrs_status wrs_table_build(wrs_table *t, const void *d_weights, uint64_t n,
 /* Build options.  The table does not depend on any of them (Alg. 3 gives
  * Alg. 2's table for every split count, Sec. 4.2); they choose how the work
  * is cut and which exact arithmetic the pack uses.
- *   splits  number of subproblems of Alg. 3's pack (one per block of the
- *           sweep, each a run of consecutive 2048-weight tiles); 0: the
- *           library's choice (8 tiles per subproblem); at most the number
- *           of tiles, ceil(n / 2048)
- *   tile    0 or 2048 (the tile is fixed)
- *   window  0 or 2048: the sweep merges a subproblem's lights with the
- *           heavy items of one stream tile at a time (its window; fixed)
+ *   splits  number of subproblems of Alg. 3's pack, each a run of
+ *           consecutive 2048-weight tiles; 0: the library's choice; at most
+ *           the number of tiles, ceil(n / 2048).  A run is packed by one warp
+ *           of the sweep, or by several where the runs are longer than eight
+ *           tiles or too few to fill the GPU
+ *   tile    0 or 2048 (fixed)
+ *   window  0 or 2048 (fixed)
  *   acc     WRS_ACC_AUTO: 64-bit bucket arithmetic when Q < 2^64, else
  *           128-bit; WRS_ACC_U64: the build fails with WRS_EOVERFLOW (in
  *           the status word) when Q >= 2^64; WRS_ACC_U128: 128-bit
@@ -261,7 +261,7 @@ wrs_status wrs_table_check_failures(const wrs_table *t, uint64_t *failures);
 uint32_t wrs_set_wait_limit(uint32_t polls);
 
 /* Test hook: during the next build, block `tile` of the look-back scan (it
- * covers 256 tiles of 2048 weights) publishes nothing, so its successor's
+ * covers 256 tiles) publishes nothing, so its successor's
  * bounded wait runs out and the build ends with WRS_ETIMEOUT instead of
  * waiting forever.  -1 (the default) disables it.  For failure-detection
  * tests only. */
@@ -338,8 +338,9 @@ wrs_status wrs_batch_download(const wrs_batch *b, void *h_buckets, uint64_t byte
 
 /* Autotuning of the sweep.  Tables fall in WRS_BATCH_CLASSES size classes by
  * tiles of 2048 weights (1, 2-4, 5-32, 33-256, more); within a class every
- * sweep block takes `group` consecutive tiles of one table (the number of
- * split subproblems of a table is its tiles / group).  wrs_batch_tune builds
+ * sweep warp takes `group` consecutive tiles of one table, at most 8 (the
+ * number of split subproblems of a table is its tiles / group; a batch of at
+ * most 2^22 weights in all is cut into tiles of 256).  wrs_batch_tune builds
  * the batch from d_weights, then for each class present times the sweep
  * with group 1, 2, 4 and 8 (best of three each, CUDA events) and keeps the
  * fastest; finally it rebuilds with the chosen groups and writes the tuned
@@ -471,7 +472,7 @@ wrs_status wrs_table2_sample_os(wrs_table2 *t, const void *d_weights, wrs_dtype 
  * back -- this entry point builds the same table as wrs_table_build
  * (bucket for bucket) into memory the caller owns, and keeps its scratch in
  * one static device array inside the library, sized for WRS_NOALLOC_MAX_N
- * weights (about 0.5 MB; every GPU that loads the library holds it until the
+ * weights (about 2.7 MB; every GPU that loads the library holds it until the
  * process exits).  It allocates nothing and calls no allocating routine.
  *
  *   d_weights  n words of dtype, device memory, 4-byte aligned, read only
@@ -506,7 +507,7 @@ typedef struct {
     uint64_t q_lo, q_hi;  /* Q */
     uint64_t qp;          /* Q >> shift: the sampler's coin denominator */
     uint32_t light_max;   /* light iff raw word <= light_max */
-    uint32_t f32;         /* library: 1 if the weights were binary32 words */
+    uint32_t f32;         /* library: how the build reads the words */
     uint64_t n;
     uint64_t n_light;
     uint64_t reserved2[8]; /* [0], [1]: zero after a build of libwrs.so; the

@@ -25,7 +25,7 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-shared"
 # (binary64 arithmetic) follow the written steps exactly.
 EXTRA = {"libwrs.so": ["-fmad=false"], "libwrs_check.so": ["-fmad=false", "-DWRS_CHECK=1"]}
 
-_WRS_HEADERS = ["wrs_device.cuh", "wrs_kernels.cuh", "wrs_batch.cuh", "wrs_twolevel.cuh", "wrs_osnd.cuh",
+_WRS_HEADERS = ["wrs_device.cuh", "wrs_pack.cuh", "wrs_kernels.cuh", "wrs_batch.cuh", "wrs_twolevel.cuh", "wrs_osnd.cuh",
                 "wrs_psaplus.cuh"]
 TARGETS = {
     "libwrs.so": (["wrs.cu"], _WRS_HEADERS, [os.path.join(INCLUDE, "wrs.h")]),

@@ -34,7 +34,6 @@ struct OpLog {
 struct wrs_table {
     uint64_t cap;          // capacity in weights
     uint64_t n;            // weights of the last build (0: never built)
-    uint32_t ntiles_cap;
     uint32_t epoch;        // look-back flag generation
     int device;
     uint8_t *ws;           // workspace block
@@ -44,7 +43,7 @@ struct wrs_table {
     TileSum *cagg, *cincl;      // per look-back chunk (256 tiles)
     uint32_t *flags;            // per chunk
     Split *split;
-    uint16_t *slist;            // per tile, kSparse offsets
+    uint16_t *slist;            // per tile, kSparseOf(tile) offsets
     uint4 *buckets;        // wrs_bucket[cap]
     void *stage_w;         // host-API staging (weights), bytes = stage_w_bytes
     uint64_t stage_w_bytes;
@@ -73,7 +72,7 @@ struct Layout {
     uint64_t hdr, part, agg, incl, cagg, cincl, flags, split, slist, total;
 };
 
-Layout layout_for(uint32_t ntiles)
+Layout layout_for(uint32_t ntiles, uint64_t slist_bytes)
 {
     const uint32_t nchunks = (ntiles + kScanChunk - 1) / kScanChunk;
     Layout L;
@@ -85,8 +84,8 @@ Layout layout_for(uint32_t ntiles)
     L.cagg = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
     L.cincl = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
     L.flags = o; o = align_up(o + (uint64_t)nchunks * sizeof(uint32_t), 256);
-    L.split = o; o = align_up(o + (uint64_t)ntiles * sizeof(Split), 256);
-    L.slist = o; o = align_up(o + (uint64_t)ntiles * kSparse * sizeof(uint16_t), 256);
+    L.split = o; o = align_up(o + ((uint64_t)ntiles + 1) * sizeof(Split), 256);
+    L.slist = o; o = align_up(o + slist_bytes, 256);
     L.total = o;
     return L;
 }
@@ -123,6 +122,39 @@ int sm_count()
     return sms > 0 ? sms : 1;
 }
 
+// Tiles of n weights: kFineTile weights each up to kFineMax (below, a sweep
+// warp per 2048 weights leaves most of the GPU idle: n = 10^6 has 489 of them
+// for 3648 resident warps), else kTile.
+inline bool fine_tiles(uint64_t n) { return n <= kFineMax; }
+inline uint32_t tile_count(uint64_t n)
+{
+    const uint64_t tile = fine_tiles(n) ? kFineTile : kTile;
+    return (uint32_t)((n + tile - 1) / tile);
+}
+// Most tiles, and list bytes, that a build of at most `cap` weights has.
+inline uint32_t tiles_cap(uint64_t cap)
+{
+    const uint32_t fine = tile_count(cap < kFineMax ? cap : kFineMax);
+    const uint32_t all = tile_count(cap);
+    return fine > all ? fine : all;
+}
+inline uint64_t slist_cap(uint64_t cap)
+{
+    const uint64_t fine = (uint64_t)tile_count(cap < kFineMax ? cap : kFineMax) * kSparseOf(kFineTile);
+    const uint64_t all = fine_tiles(cap) ? fine : (uint64_t)tile_count(cap) * kSparseOf(kTile);
+    return (fine > all ? fine : all) * sizeof(uint16_t);
+}
+
+// Own tiles per task of the sweep (a warp each), at most `most`: as many as
+// leave every resident warp four tasks.
+uint32_t sweep_group(uint32_t ntiles, uint32_t most)
+{
+    const uint64_t want = 4ull * kPackBlocks * (uint64_t)sm_count();
+    uint32_t g = kSweepTiles;
+    while (g > 1 && (g > most || ntiles / g < want)) g /= 2;
+    return g;
+}
+
 std::atomic<bool> g_attr_done[64];
 std::mutex g_attr_mu;
 
@@ -133,9 +165,10 @@ wrs_status set_kernel_attributes()
     if (g_attr_done[dev].load(std::memory_order_acquire)) return WRS_OK;
     std::lock_guard<std::mutex> lock(g_attr_mu);
     if (g_attr_done[dev].load(std::memory_order_relaxed)) return WRS_OK;
-    const int bytes = (int)sizeof(SweepSmem);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sweep<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    const int bytes = (int)kPackSmemBytes;
+    cudaError_t e = cudaSuccess;
+    for (auto *k : {k_sweep<0, kTile>, k_sweep<1, kTile>, k_sweep<0, kFineTile>, k_sweep<1, kFineTile>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return WRS_EDEVICE;
     g_attr_done[dev].store(true, std::memory_order_release);
     return WRS_OK;
@@ -226,6 +259,29 @@ struct BuildOpts {
     int acc = WRS_ACC_AUTO;
 };
 
+void launch_classify(uint32_t blocks, cudaStream_t s, bool f32, bool fine, const uint32_t *w, uint64_t n, int vec,
+                     const DevHeader *hdr, TileSum *agg, uint16_t *slist, uint32_t ntiles)
+{
+    auto *k = f32 ? (fine ? k_classify<1, kFineTile> : k_classify<1, kTile>)
+                  : (fine ? k_classify<0, kFineTile> : k_classify<0, kTile>);
+    k<<<blocks, kThreads, 0, s>>>(w, n, vec, hdr, agg, slist, ntiles);
+}
+
+void launch_split(cudaStream_t s, bool fine, const TileSum *incl, uint32_t ntiles, uint64_t n, DevHeader *hdr,
+                  Split *split)
+{
+    auto *k = fine ? k_split<kFineTile> : k_split<kTile>;
+    k<<<ntiles / kThreads + 1, kThreads, 0, s>>>(incl, ntiles, n, hdr, split); // one boundary more than tiles
+}
+
+void launch_sweep(cudaStream_t s, bool f32, bool fine, const uint32_t *w, uint64_t n, int vec, DevHeader *hdr,
+                  const Split *split, const uint16_t *slist, uint32_t ntiles, uint4 *table, uint32_t group, int wide)
+{
+    auto *k = f32 ? (fine ? k_sweep<1, kFineTile> : k_sweep<1, kTile>)
+                  : (fine ? k_sweep<0, kFineTile> : k_sweep<0, kTile>);
+    k<<<(ntiles + group - 1) / group, 32, kPackSmemBytes, s>>>(w, n, vec, hdr, split, slist, ntiles, table, group, wide);
+}
+
 wrs_status enqueue_build(wrs_table *t, const void *d_weights, uint64_t n, wrs_dtype dtype, cudaStream_t s,
                          const BuildOpts &o = BuildOpts())
 {
@@ -235,7 +291,8 @@ wrs_status enqueue_build(wrs_table *t, const void *d_weights, uint64_t n, wrs_dt
     }
     const uint32_t *w = static_cast<const uint32_t *>(d_weights);
     const int vec = (reinterpret_cast<uintptr_t>(w) % 16) == 0;
-    const uint32_t ntiles = (uint32_t)((n + kTile - 1) / kTile);
+    const uint32_t ntiles = tile_count(n);
+    const bool fine = fine_tiles(n);
     const uint32_t f32 = dtype == WRS_F32;
     uint64_t want = (n + (uint64_t)kThreads * 16 - 1) / ((uint64_t)kThreads * 16);
     uint32_t nparts = (uint32_t)(want < 1 ? 1 : (want > kMaxParts ? kMaxParts : want));
@@ -263,20 +320,17 @@ wrs_status enqueue_build(wrs_table *t, const void *d_weights, uint64_t n, wrs_dt
     if (tm) cudaEventRecord(t->ev[1], s);
     k_stats_combine<<<1, kThreads, 0, s>>>(t->part, nparts, n, f32, t->hdr);
     if (tm) cudaEventRecord(t->ev[2], s);
-    if (f32) k_classify<1><<<cls_blocks, kThreads, 0, s>>>(w, n, vec, t->hdr, t->agg, t->slist, ntiles);
-    else k_classify<0><<<cls_blocks, kThreads, 0, s>>>(w, n, vec, t->hdr, t->agg, t->slist, ntiles);
+    launch_classify(cls_blocks, s, f32, fine, w, n, vec, t->hdr, t->agg, t->slist, ntiles);
     if (tm) cudaEventRecord(t->ev[3], s);
     k_tilescan<<<nchunks, kThreads, 0, s>>>(t->hdr, t->agg, t->cagg, t->cincl, t->incl, t->flags, ntiles, epoch,
                                             wait_limit, skip_tile);
     if (tm) cudaEventRecord(t->ev[4], s);
-    k_split<<<(ntiles + kThreads - 1) / kThreads, kThreads, 0, s>>>(t->incl, ntiles, n, t->hdr, t->split);
+    launch_split(s, fine, t->incl, ntiles, n, t->hdr, t->split);
     if (o.acc == WRS_ACC_U64) k_require_u64<<<1, 32, 0, s>>>(t->hdr);
     if (tm) cudaEventRecord(t->ev[5], s);
-    const size_t sweep_smem = sizeof(SweepSmem);
-    const uint32_t sweep_blocks = (ntiles + o.group - 1) / o.group;
-    const int wide = o.acc == WRS_ACC_U128;
-    if (f32) k_sweep<1><<<sweep_blocks, kThreads, sweep_smem, s>>>(w, n, vec, t->hdr, t->incl, t->split, t->slist, ntiles, t->buckets, o.group, wide);
-    else k_sweep<0><<<sweep_blocks, kThreads, sweep_smem, s>>>(w, n, vec, t->hdr, t->incl, t->split, t->slist, ntiles, t->buckets, o.group, wide);
+    // a subproblem of the caller's split count (a run of tiles) is packed by one or more warps
+    const uint32_t group = sweep_group(ntiles, fine ? o.group * (kTile / kFineTile) : o.group);
+    launch_sweep(s, f32, fine, w, n, vec, t->hdr, t->split, t->slist, ntiles, t->buckets, group, o.acc == WRS_ACC_U128);
     if (tm) cudaEventRecord(t->ev[6], s);
     t->timed_build = tm;
     wrs_status st = launch_err();
@@ -332,10 +386,9 @@ wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out)
     t->log = new (std::nothrow) OpLog();
     if (!t->log) { delete t; return WRS_ENOMEM; }
     t->cap = capacity_n;
-    t->ntiles_cap = (uint32_t)((capacity_n + kTile - 1) / kTile);
     t->host_status = -1;
     cudaGetDevice(&t->device);
-    const Layout L = layout_for(t->ntiles_cap);
+    const Layout L = layout_for(tiles_cap(capacity_n), slist_cap(capacity_n));
     cudaError_t e = cudaStreamCreateWithFlags(&t->log->priv, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->log->build_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) { destroy_log(t->log); delete t; return cuda_err(e); }
@@ -684,7 +737,8 @@ void wrs_debug_skip_publish(int64_t tile)
 namespace {
 
 constexpr uint64_t kNaMaxN = WRS_NOALLOC_MAX_N;
-constexpr uint32_t kNaTiles = (uint32_t)((kNaMaxN + kTile - 1) / kTile);
+static_assert(kNaMaxN <= kFineMax, "the static scratch holds fine tiles");
+constexpr uint32_t kNaTiles = (uint32_t)((kNaMaxN + kFineTile - 1) / kFineTile);
 constexpr uint32_t kNaChunks = (kNaTiles + kScanChunk - 1) / kScanChunk;
 constexpr uint64_t na_up(uint64_t x) { return (x + 255) / 256 * 256; }
 constexpr uint64_t kNaPart = 0;
@@ -694,8 +748,8 @@ constexpr uint64_t kNaCagg = kNaIncl + na_up((uint64_t)kNaTiles * sizeof(TileSum
 constexpr uint64_t kNaCincl = kNaCagg + na_up((uint64_t)kNaChunks * sizeof(TileSum));
 constexpr uint64_t kNaFlags = kNaCincl + na_up((uint64_t)kNaChunks * sizeof(TileSum));
 constexpr uint64_t kNaSplit = kNaFlags + na_up((uint64_t)kNaChunks * sizeof(uint32_t));
-constexpr uint64_t kNaSlist = kNaSplit + na_up((uint64_t)kNaTiles * sizeof(Split));
-constexpr uint64_t kNaBytes = kNaSlist + na_up((uint64_t)kNaTiles * kSparse * sizeof(uint16_t));
+constexpr uint64_t kNaSlist = kNaSplit + na_up(((uint64_t)kNaTiles + 1) * sizeof(Split));
+constexpr uint64_t kNaBytes = kNaSlist + na_up((uint64_t)kNaTiles * kSparseOf(kFineTile) * sizeof(uint16_t));
 
 // Zero at module load.  Every call clears the look-back flags on its stream
 // before the scan and publishes with generation 1, so nothing on the launch
@@ -755,7 +809,7 @@ extern "C" wrs_status wrs_build_noalloc(const void *d_weights, uint64_t n, wrs_d
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const uint32_t *w = static_cast<const uint32_t *>(d_weights);
     const int vec = (reinterpret_cast<uintptr_t>(w) % 16) == 0;
-    const uint32_t ntiles = (uint32_t)((n + kTile - 1) / kTile);
+    const uint32_t ntiles = tile_count(n);
     const uint32_t nchunks = (ntiles + kScanChunk - 1) / kScanChunk;
     const uint32_t f32 = dtype == WRS_F32;
     DevHeader *hdr = static_cast<DevHeader *>(d_header);
@@ -783,14 +837,11 @@ extern "C" wrs_status wrs_build_noalloc(const void *d_weights, uint64_t n, wrs_d
     if (f32) k_stats<1><<<nparts, kThreads, 0, s>>>(w, n, vec, part);
     else k_stats<0><<<nparts, kThreads, 0, s>>>(w, n, vec, part);
     k_stats_combine<<<1, kThreads, 0, s>>>(part, nparts, n, f32, hdr);
-    if (f32) k_classify<1><<<cls_blocks, kThreads, 0, s>>>(w, n, vec, hdr, agg, slist, ntiles);
-    else k_classify<0><<<cls_blocks, kThreads, 0, s>>>(w, n, vec, hdr, agg, slist, ntiles);
+    launch_classify(cls_blocks, s, f32, true, w, n, vec, hdr, agg, slist, ntiles);
     k_tilescan<<<nchunks, kThreads, 0, s>>>(hdr, agg, cagg, cincl, incl, flags, ntiles, kNaEpoch,
                                             g_wait_limit.load(), kNone);
-    k_split<<<(ntiles + kThreads - 1) / kThreads, kThreads, 0, s>>>(incl, ntiles, n, hdr, split);
-    const uint32_t sweep_blocks = (ntiles + kSweepTiles - 1) / kSweepTiles;
-    if (f32) k_sweep<1><<<sweep_blocks, kThreads, sizeof(SweepSmem), s>>>(w, n, vec, hdr, incl, split, slist, ntiles, buckets, kSweepTiles, 0);
-    else k_sweep<0><<<sweep_blocks, kThreads, sizeof(SweepSmem), s>>>(w, n, vec, hdr, incl, split, slist, ntiles, buckets, kSweepTiles, 0);
+    launch_split(s, true, incl, ntiles, n, hdr, split);
+    launch_sweep(s, f32, true, w, n, vec, hdr, split, slist, ntiles, buckets, sweep_group(ntiles, kSweepTiles), 0);
     return launch_err();
 }
 

@@ -39,8 +39,9 @@ constexpr int kBatchClasses = WRS_BATCH_CLASSES; // sweep size classes by tiles:
 constexpr uint32_t kBatchGroups[] = {1, 2, 4, 8}; // tuner's candidates for own tiles per sweep block
 constexpr uint32_t kBatchPartWeights = 16384;    // weights per k_stats block (at least)
 
-inline int batch_class(uint32_t ntiles)
+inline int batch_class(uint64_t n)
 {
+    const uint64_t ntiles = (n + kTile - 1) / kTile;
     return ntiles <= 1 ? 0 : ntiles <= 4 ? 1 : ntiles <= 32 ? 2 : ntiles <= 256 ? 3 : 4;
 }
 
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(kThreads) kb_stats(const uint32_t *__restrict_
 }
 
 // One block per table; block 0 also advances the look-back generation.
-// Tables of one tile are built by kb_small instead.
+// Tables of at most kTile weights are built by kb_small instead.
 __global__ void __launch_bounds__(kThreads) kb_stats_combine(const BatchTable *__restrict__ bt,
                                                              const Partial *__restrict__ part, uint32_t f32,
                                                              DevHeader *hdr, uint32_t *epoch)
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kThreads) kb_stats_combine(const BatchTable *_
         *epoch = e;
     }
     const BatchTable &T = bt[blockIdx.x];
-    if (T.ntiles <= 1) return;
+    if (T.n <= (uint64_t)kTile) return;
     stats_combine_body(part + T.part0, T.nparts, T.n, f32, hdr + blockIdx.x);
 }
 
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restri
     a.base = F32 ? INT_MAX : 0;
     a.acc = 0;
     a.flags = 0;
+    a.mx = 0;
     uint64_t a64 = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restri
     if (bad) set_status(hdr, kEInternal);
 }
 
-template <int F32>
+template <int F32, int TILE>
 __global__ void __launch_bounds__(kThreads) kb_classify(const uint32_t *__restrict__ w, int vec,
                                                         const BatchTable *__restrict__ bt,
                                                         const BlockMap *__restrict__ map, const DevHeader *hdr,
@@ -136,7 +138,8 @@ __global__ void __launch_bounds__(kThreads) kb_classify(const uint32_t *__restri
 {
     const BlockMap m = map[blockIdx.x]; // block m.local: tiles 8 m.local .. 8 m.local + 7, one per warp
     const BatchTable &T = bt[m.table];
-    classify_body<F32>(w + T.off, T.n, vec, hdr + m.table, agg + T.tile0, slist + (uint64_t)T.tile0 * kSparse,
+    classify_body<F32, TILE>(w + T.off, T.n, vec, hdr + m.table, agg + T.tile0,
+                             slist + (uint64_t)T.tile0 * kSparseOf(TILE),
                        T.ntiles, m.local * kWarps + (threadIdx.x >> 5), T.ntiles);
 }
 
@@ -152,6 +155,7 @@ __global__ void __launch_bounds__(kThreads) kb_tilescan(const BatchTable *__rest
                   flags + T.chunk0, T.ntiles, __ldcg(epoch), wait_limit, kNone);
 }
 
+template <int TILE>
 __global__ void __launch_bounds__(kThreads) kb_split(const BatchTable *__restrict__ bt,
                                                      const BlockMap *__restrict__ map,
                                                      const TileSum *__restrict__ incl, DevHeader *hdr,
@@ -159,22 +163,22 @@ __global__ void __launch_bounds__(kThreads) kb_split(const BatchTable *__restric
 {
     const BlockMap m = map[blockIdx.x];
     const BatchTable &T = bt[m.table];
-    split_body(incl + T.tile0, T.ntiles, T.n, hdr + m.table, split + T.tile0, m.local * kThreads + threadIdx.x);
+    split_body<TILE>(incl + T.tile0, T.ntiles, T.n, hdr + m.table, split + T.tile0 + m.table, // one boundary more than tiles
+               m.local * kThreads + threadIdx.x);
 }
 
-template <int F32>
-__global__ void __launch_bounds__(kThreads, 3) kb_sweep(const uint32_t *__restrict__ w, int vec,
+template <int F32, int TILE>
+__global__ void __launch_bounds__(32, kPackBlocks) kb_sweep(const uint32_t *__restrict__ w, int vec,
                                                         const BatchTable *__restrict__ bt,
                                                         const BlockMap *__restrict__ map, DevHeader *hdr,
-                                                        const TileSum *__restrict__ incl,
                                                         const Split *__restrict__ split,
                                                         const uint16_t *__restrict__ slist, uint4 *__restrict__ buckets)
 {
     const BlockMap m = map[blockIdx.x];
     const BatchTable &T = bt[m.table];
     const uint32_t c_first = m.local * T.group;
-    sweep_body<F32>(w + T.off, T.n, vec, hdr + m.table, incl + T.tile0, split + T.tile0,
-                    slist + (uint64_t)T.tile0 * kSparse, T.ntiles, buckets + T.off, c_first,
+    sweep_body<F32, TILE>(w + T.off, T.n, vec, hdr + m.table, split + T.tile0 + m.table,
+                    slist + (uint64_t)T.tile0 * kSparseOf(TILE), T.ntiles, buckets + T.off, c_first,
                     min(c_first + T.group, T.ntiles));
 }
 
@@ -248,6 +252,7 @@ struct wrs_batch {
     uint64_t total_k;
     std::vector<BatchTable> h;
     uint32_t groups[kBatchClasses];
+    bool fine;             // fine tiles (the same for all tables)
     uint8_t *ws;           // one allocation: tables, headers, per-part/tile/chunk arrays, epoch
     BatchTable *d_tables;
     DevHeader *hdr;
@@ -302,14 +307,22 @@ wrs_status apply_groups(wrs_batch *b)
     std::vector<BlockMap> m;
     for (uint32_t t = 0; t < b->ntables; ++t) {
         BatchTable &T = b->h[t];
-        T.group = b->groups[batch_class(T.ntiles)];
-        if (T.ntiles <= 1) continue; // built whole by kb_small
+        T.group = std::min<uint32_t>(b->groups[batch_class(T.n)], kSweepTiles);
+        if (T.n <= (uint64_t)kTile) continue; // built whole by kb_small
         const uint32_t nblk = (T.ntiles + T.group - 1) / T.group;
         for (uint32_t i = 0; i < nblk; ++i) m.push_back(BlockMap{t, i});
     }
     wrs_status st = upload_map(b, kMapSweep, m);
     if (st == WRS_OK) st = upload_tables(b);
     return st;
+}
+
+void batch_launch_sweep(wrs_batch *b, const uint32_t *w, int vec, bool f32, cudaStream_t s)
+{
+    auto *k = f32 ? (b->fine ? kb_sweep<1, kFineTile> : kb_sweep<1, kTile>)
+                  : (b->fine ? kb_sweep<0, kFineTile> : kb_sweep<0, kTile>);
+    k<<<b->nb[kMapSweep], 32, kPackSmemBytes, s>>>(w, vec, b->d_tables, b->map[kMapSweep], b->hdr, b->split, b->slist,
+                                                   b->buckets);
 }
 
 wrs_status batch_enqueue_build(wrs_batch *b, const uint32_t *w, uint32_t f32, cudaStream_t s, cudaEvent_t sweep0,
@@ -333,15 +346,15 @@ wrs_status batch_enqueue_build(wrs_batch *b, const uint32_t *w, uint32_t f32, cu
     if (f32) kb_stats<1><<<b->nb[kMapStats], kThreads, 0, s>>>(w, vec, b->d_tables, b->map[kMapStats], b->part);
     else kb_stats<0><<<b->nb[kMapStats], kThreads, 0, s>>>(w, vec, b->d_tables, b->map[kMapStats], b->part);
     kb_stats_combine<<<b->ntables, kThreads, 0, s>>>(b->d_tables, b->part, f32, b->hdr, b->epoch);
-    if (f32) kb_classify<1><<<b->nb[kMapClassify], kThreads, 0, s>>>(w, vec, b->d_tables, b->map[kMapClassify], b->hdr, b->agg, b->slist);
-    else kb_classify<0><<<b->nb[kMapClassify], kThreads, 0, s>>>(w, vec, b->d_tables, b->map[kMapClassify], b->hdr, b->agg, b->slist);
+    auto *classify = f32 ? (b->fine ? kb_classify<1, kFineTile> : kb_classify<1, kTile>)
+                         : (b->fine ? kb_classify<0, kFineTile> : kb_classify<0, kTile>);
+    classify<<<b->nb[kMapClassify], kThreads, 0, s>>>(w, vec, b->d_tables, b->map[kMapClassify], b->hdr, b->agg, b->slist);
     kb_tilescan<<<b->nb[kMapScan], kThreads, 0, s>>>(b->d_tables, b->map[kMapScan], b->hdr, b->agg, b->cagg,
                                                       b->cincl, b->incl, b->flags, b->epoch, g_wait_limit.load());
-    kb_split<<<b->nb[kMapSplit], kThreads, 0, s>>>(b->d_tables, b->map[kMapSplit], b->incl, b->hdr, b->split);
+    auto *split = b->fine ? kb_split<kFineTile> : kb_split<kTile>;
+    split<<<b->nb[kMapSplit], kThreads, 0, s>>>(b->d_tables, b->map[kMapSplit], b->incl, b->hdr, b->split);
     if (sweep0) cudaEventRecord(sweep0, s);
-    const size_t smem = sizeof(SweepSmem);
-    if (f32) kb_sweep<1><<<b->nb[kMapSweep], kThreads, smem, s>>>(w, vec, b->d_tables, b->map[kMapSweep], b->hdr, b->incl, b->split, b->slist, b->buckets);
-    else kb_sweep<0><<<b->nb[kMapSweep], kThreads, smem, s>>>(w, vec, b->d_tables, b->map[kMapSweep], b->hdr, b->incl, b->split, b->slist, b->buckets);
+    batch_launch_sweep(b, w, vec, f32, s);
     if (sweep1) cudaEventRecord(sweep1, s);
     return launch_err();
 }
@@ -350,9 +363,7 @@ wrs_status batch_enqueue_sweep(wrs_batch *b, const uint32_t *w, uint32_t f32, cu
 {
     if (b->nb[kMapSweep] == 0) return WRS_OK;
     const int vec = (reinterpret_cast<uintptr_t>(w) % 16) == 0;
-    const size_t smem = sizeof(SweepSmem);
-    if (f32) kb_sweep<1><<<b->nb[kMapSweep], kThreads, smem, s>>>(w, vec, b->d_tables, b->map[kMapSweep], b->hdr, b->incl, b->split, b->slist, b->buckets);
-    else kb_sweep<0><<<b->nb[kMapSweep], kThreads, smem, s>>>(w, vec, b->d_tables, b->map[kMapSweep], b->hdr, b->incl, b->split, b->slist, b->buckets);
+    batch_launch_sweep(b, w, vec, f32, s);
     return launch_err();
 }
 
@@ -364,9 +375,10 @@ wrs_status batch_kernel_attributes()
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return WRS_EDEVICE;
     if (g_batch_attr_done[dev]) return WRS_OK;
-    const int bytes = (int)sizeof(SweepSmem), gbytes = (int)sizeof(GroupSmem);
-    cudaError_t e = cudaFuncSetAttribute(kb_sweep<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_sweep<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    const int bytes = (int)kPackSmemBytes, gbytes = (int)sizeof(GroupSmem);
+    cudaError_t e = cudaSuccess;
+    for (auto *k : {kb_sweep<0, kTile>, kb_sweep<1, kTile>, kb_sweep<0, kFineTile>, kb_sweep<1, kFineTile>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_small<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, gbytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_small<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, gbytes);
     if (e != cudaSuccess) return WRS_EDEVICE;
@@ -410,13 +422,15 @@ wrs_status wrs_batch_create(uint32_t ntables, const uint64_t *h_n, wrs_batch **o
     b->ntables = ntables;
     b->h.resize(ntables);
     cudaGetDevice(&b->device);
+    b->fine = fine_tiles(off[ntables]); // as a single table of all these weights
+    const uint64_t tile = b->fine ? kFineTile : kTile;
     uint64_t tiles = 0, parts = 0, chunks = 0;
     for (uint32_t t = 0; t < ntables; ++t) {
         BatchTable &T = b->h[t];
         std::memset(&T, 0, sizeof(T));
         T.off = off[t];
         T.n = h_n[t];
-        T.ntiles = (uint32_t)((T.n + kTile - 1) / kTile);
+        T.ntiles = (uint32_t)((T.n + tile - 1) / tile);
         T.tile0 = (uint32_t)tiles;
         uint64_t np = (T.n + kBatchPartWeights - 1) / kBatchPartWeights;
         T.nparts = (uint32_t)std::min<uint64_t>(np, (uint64_t)sm_count() * 8);
@@ -431,7 +445,7 @@ wrs_status wrs_batch_create(uint32_t ntables, const uint64_t *h_n, wrs_batch **o
     b->total_tiles = (uint32_t)tiles;
     b->total_parts = (uint32_t)parts;
     b->total_chunks = (uint32_t)chunks;
-    for (int c = 0; c < kBatchClasses; ++c) b->groups[c] = c == 0 ? 1 : kSweepTiles;
+    for (int c = 0; c < kBatchClasses; ++c) b->groups[c] = c == 0 ? 1 : sweep_group(b->total_tiles, kSweepTiles);
 
     uint64_t o = 0;
     auto carve = [&](uint64_t bytes) { const uint64_t at = o; o = align_up(o + bytes, 256); return at; };
@@ -443,8 +457,8 @@ wrs_status wrs_batch_create(uint32_t ntables, const uint64_t *h_n, wrs_batch **o
     const uint64_t o_cagg = carve(chunks * sizeof(TileSum));
     const uint64_t o_cincl = carve(chunks * sizeof(TileSum));
     const uint64_t o_flags = carve(chunks * sizeof(uint32_t));
-    const uint64_t o_split = carve(tiles * sizeof(Split));
-    const uint64_t o_slist = carve(tiles * kSparse * sizeof(uint16_t));
+    const uint64_t o_split = carve((tiles + ntables) * sizeof(Split));
+    const uint64_t o_slist = carve(tiles * kSparseOf((int)tile) * sizeof(uint16_t));
     const uint64_t o_epoch = carve(sizeof(uint32_t));
     cudaError_t e = cudaMalloc(&b->ws, o);
     if (e != cudaSuccess) { delete b; return cuda_err(e); }
@@ -467,11 +481,11 @@ wrs_status wrs_batch_create(uint32_t ntables, const uint64_t *h_n, wrs_batch **o
     std::vector<BlockMap> ms, msmall, mc, mscan, msplit;
     for (uint32_t t = 0; t < ntables; ++t) {
         const BatchTable &T = b->h[t];
-        if (T.ntiles <= 1) { msmall.push_back(BlockMap{t, 0}); continue; } // one block builds it whole
+        if (T.n <= (uint64_t)kTile) { msmall.push_back(BlockMap{t, 0}); continue; } // one block builds it whole
         for (uint32_t i = 0; i < T.nparts; ++i) ms.push_back(BlockMap{t, i});
         for (uint32_t i = 0; i < (T.ntiles + kWarps - 1) / kWarps; ++i) mc.push_back(BlockMap{t, i});
         for (uint32_t i = 0; i < (T.ntiles + kScanChunk - 1) / kScanChunk; ++i) mscan.push_back(BlockMap{t, i});
-        for (uint32_t i = 0; i < (T.ntiles + kThreads - 1) / kThreads; ++i) msplit.push_back(BlockMap{t, i});
+        for (uint32_t i = 0; i < (T.ntiles + kThreads) / kThreads; ++i) msplit.push_back(BlockMap{t, i});
     }
     st = upload_map(b, kMapStats, ms);
     if (st == WRS_OK) st = upload_map(b, kMapSmall, msmall);
@@ -611,7 +625,7 @@ wrs_status wrs_batch_tune(wrs_batch *b, const void *d_weights, wrs_dtype dtype, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     bool present[kBatchClasses] = {};
     for (const BatchTable &T : b->h)
-        if (T.ntiles > 1) present[batch_class(T.ntiles)] = true; // one-tile tables: kb_small, no sweep
+        if (T.n > (uint64_t)kTile) present[batch_class(T.n)] = true; // kb_small's tables have no sweep
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         if (e0) cudaEventDestroy(e0);

@@ -16,7 +16,12 @@ constexpr int kTile = kThreads * kItems;    // weights per tile (2048)
 constexpr int kWarps = kThreads / 32;
 constexpr int kChunk = 32 * kItems;         // weights of one warp's share of a tile (256)
 constexpr int kChunks = kTile / kChunk;     // chunks per tile (8)
-constexpr int kSparse = 32;                 // member lists of tiles with <= 32 heavies (or lights)
+// The build's split granularity: tiles of kTile weights, or of kFineTile when
+// the weights are too few for a warp of the sweep per large tile to fill the
+// GPU.  Tiles with at most kSparseOf(tile) heavies have a list of them.
+constexpr int kFineTile = kChunk;
+constexpr uint64_t kFineMax = 1ull << 22;   // weights up to which fine tiles are used
+__host__ __device__ constexpr int kSparseOf(int tile) { return tile == kFineTile ? 8 : 32; }
 constexpr int kScanChunk = kThreads;        // tile aggregates per block of the look-back scan
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kQBits = 95;                  // Q < 2^95 keeps n*Q < 2^127
@@ -35,7 +40,7 @@ struct DevHeader {
     uint64_t q_lo, q_hi;    // Q
     uint64_t qp;            // Q >> shift
     uint32_t light_max;     // light iff raw word <= light_max
-    uint32_t f32;
+    uint32_t f32;           // bit 0: binary32 weights; bits 8 and up: the sweep's PackMode
     uint64_t n;
     uint64_t n_light;       // filled by the sweep of the last tile
     uint64_t pad[2];        // zero; the check build counts failed checks in pad[0]
@@ -45,7 +50,7 @@ struct Partial {            // per-block result of k_stats
     uint64_t lo, hi;        // exact partial sum (units of 2^base)
     int32_t base;           // INT_MAX: no nonzero weight seen
     uint32_t flags;         // bit 0 invalid weight, bit 1 range exceeded
-    uint64_t pad;
+    uint32_t mx, pad;       // largest word
 };
 constexpr uint32_t kPartInvalid = 1u, kPartOverflow = 2u;
 
@@ -58,12 +63,13 @@ struct TileSum {            // per-tile aggregate, or inclusive prefix over tile
     uint32_t pad;
 };
 
-struct Split {              // per-tile result of k_split
-    uint32_t hb;            // tile holding the heavy current at this tile's first light
-    uint32_t lb;            // a tile at or before the one holding the light that follows
-                            // this tile's first heavy
+struct Split {              // result of k_split per tile boundary (48 B; ntiles + 1 of them)
+    uint32_t hb;            // tile holding the heavy current at the first light from this tile on
     uint32_t next_heavy;    // position of the first heavy item after this tile
-    uint32_t pad;
+    uint32_t nheavy;        // heavy items in this tile
+    uint32_t ch;            // heavy items before this tile
+    uint64_t d_lo, d_hi;    // D of the first light from this tile on
+    uint64_t e_lo, e_hi;    // E after the heavies before this tile
 };
 
 // ------------------------------------------------------------ 128-bit ops

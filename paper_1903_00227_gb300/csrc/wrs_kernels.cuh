@@ -4,15 +4,16 @@
 // Build (alias table of n weights; Alg. 3 "PSA", Sec. 4.2, producing the
 // table of Alg. 2, Sec. 4.1, bucket for bucket):
 //   k_stats, k_stats_combine  W := sum w_i, exactly (opening line of Alg. 3)
-//   k_classify  per 2048-weight tile: light/heavy classification (Alg. 3's
+//   k_classify  per tile of 2048 (or 256) weights: light/heavy classification (Alg. 3's
 //               two traversals) and the tile's light and heavy weight sums
 //               and counts (Sec. 4.2.2 "Using Block-Wise Prefix Sums": tiles
 //               play the role of the blocks), plus the offsets of the tile's
-//               members of a class that has at most 32 of them
+//               heavies when they are few
 //   k_tilescan  inclusive prefix of the tile aggregates: a single-pass scan
 //               with decoupled look-back between thread blocks
 //   k_split     per tile, Alg. 3's split search on the tile prefix sums
-//   k_sweep     per tile, the buckets of the tile's own items (Alg. 3's pack)
+//   k_sweep     per run of tiles, the buckets of its lights and the heavies packed
+//               with them (Alg. 3's pack)
 // Query:
 //   k_sample    k alias queries (Sec. 2.2; Sec. 5 Cor. "kWR"), branchless
 //               selection between bucket and alias (Sec. 10, "Optimizations").
@@ -30,6 +31,7 @@
 #pragma once
 
 #include "wrs_device.cuh"
+#include "wrs_pack.cuh"
 
 namespace wrs {
 
@@ -74,11 +76,13 @@ struct Acc {
     int base;
     u128 acc;
     uint32_t flags;
+    uint32_t mx;     // largest word
 };
 
 __device__ __forceinline__ void acc_merge(Acc &a, const Acc &b)
 {
     a.flags |= b.flags;
+    a.mx = max(a.mx, b.mx);
     if (b.base == INT_MAX) return;
     if (a.base == INT_MAX) { a.base = b.base; a.acc = b.acc; return; }
     u128 lo_acc = a.acc, hi_acc = b.acc;
@@ -100,6 +104,7 @@ __device__ __forceinline__ void acc_take(Acc &a, uint64_t &a64, uint32_t x)
 {
     if (!F32) { a64 += x; return; }
     const uint32_t ex = (x >> 23) & 0xFFu;
+    a.mx = max(a.mx, x);
     if ((x >> 31) || ex == 0xFFu) { a.flags |= kPartInvalid; return; }
     uint32_t m = x & 0x7FFFFFu;
     if (ex) m |= 0x800000u;
@@ -138,6 +143,7 @@ __device__ __forceinline__ Acc acc_shfl_down(const Acc &a, int d)
     b.base = __shfl_down_sync(0xFFFFFFFFu, a.base, d);
     b.acc = shfl_down128(a.acc, d);
     b.flags = __shfl_down_sync(0xFFFFFFFFu, a.flags, d);
+    b.mx = __shfl_down_sync(0xFFFFFFFFu, a.mx, d);
     return b;
 }
 
@@ -145,19 +151,19 @@ __device__ Acc acc_block_reduce(Acc a)
 {
     __shared__ int s_base[kWarps];
     __shared__ u128 s_acc[kWarps];
-    __shared__ uint32_t s_flags[kWarps];
+    __shared__ uint32_t s_flags[kWarps], s_mx[kWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
         Acc b = acc_shfl_down(a, d);
         acc_merge(a, b);
     }
-    if (lane == 0) { s_base[wid] = a.base; s_acc[wid] = a.acc; s_flags[wid] = a.flags; }
+    if (lane == 0) { s_base[wid] = a.base; s_acc[wid] = a.acc; s_flags[wid] = a.flags; s_mx[wid] = a.mx; }
     __syncthreads();
     if (wid == 0) {
         Acc b;
-        if (lane < kWarps) { b.base = s_base[lane]; b.acc = s_acc[lane]; b.flags = s_flags[lane]; }
-        else { b.base = INT_MAX; b.acc = 0; b.flags = 0; }
+        if (lane < kWarps) { b.base = s_base[lane]; b.acc = s_acc[lane]; b.flags = s_flags[lane]; b.mx = s_mx[lane]; }
+        else { b.base = INT_MAX; b.acc = 0; b.flags = 0; b.mx = 0; }
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
             Acc c = acc_shfl_down(b, d);
@@ -203,6 +209,7 @@ __device__ __forceinline__ void stats_body(const uint32_t *__restrict__ w, uint6
     a.base = F32 ? INT_MAX : 0;
     a.acc = 0;
     a.flags = 0;
+    a.mx = 0; // not needed for integer weights
     uint64_t a64 = 0;
     if (!F32) {
         const uint64_t tid = (uint64_t)bid * kThreads + threadIdx.x;
@@ -275,11 +282,12 @@ __device__ __forceinline__ void stats_body(const uint32_t *__restrict__ w, uint6
             }
         }
         if (vmax >= 0x7F800000u) a.flags |= kPartInvalid;
+        a.mx = max(a.mx, vmax);
     }
     a = acc_block_reduce(a);
     if (threadIdx.x == 0) {
         Partial p;
-        p.lo = lo64(a.acc); p.hi = hi64(a.acc); p.base = a.base; p.flags = a.flags; p.pad = 0;
+        p.lo = lo64(a.acc); p.hi = hi64(a.acc); p.base = a.base; p.flags = a.flags; p.mx = a.mx; p.pad = 0;
         *out = p;
     }
 }
@@ -314,11 +322,11 @@ __device__ __forceinline__ void stats_combine_body(const Partial *__restrict__ p
                                                    uint32_t f32, DevHeader *hdr)
 {
     Acc a;
-    a.base = INT_MAX; a.acc = 0; a.flags = 0;
+    a.base = INT_MAX; a.acc = 0; a.flags = 0; a.mx = 0;
     for (uint32_t i = threadIdx.x; i < nparts; i += kThreads) {
         Partial p = part[i];
         Acc b;
-        b.base = p.base; b.acc = mk128(p.lo, p.hi); b.flags = p.flags;
+        b.base = p.base; b.acc = mk128(p.lo, p.hi); b.flags = p.flags; b.mx = p.mx;
         if (!f32) b.base = 0;
         acc_merge(a, b);
     }
@@ -358,7 +366,14 @@ __device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint3
     hdr->q_hi = hi64(Q);
     hdr->qp = lo64(Q >> shift);
     hdr->light_max = light_max;
-    hdr->f32 = f32;
+    // how the sweep forms n q and its keys (PackMode)
+    uint32_t mode = kPackQ128;
+    if (shift == 0 && bitlen128(Q) + (32 - __clz((int)(uint32_t)n)) <= 95) {
+        const bool normal = !f32 || beta >= -94;
+        if (normal && (!f32 || (int)(a.mx >> 23) <= 158 + beta)) mode = kPackQ32;
+        else if (normal && (int)(light_max >> 23) <= 158 + beta) mode = kPackQ96;
+    }
+    hdr->f32 = f32 | mode << 8;
     hdr->n = n;
     hdr->n_light = 0;
     hdr->pad[0] = 0;
@@ -437,16 +452,17 @@ __device__ __forceinline__ uint32_t warp_excl_scan_u32(uint32_t v)
 }
 
 // Tiles t_first, t_first + t_stride, ... of one table, ONE WARP per tile
-// (no block barrier per tile).  A tile is eight chunks of 256 weights; lane
+// (no block barrier per tile).  A tile is TILE / 256 chunks of 256 weights; lane
 // l holds weights 8l .. 8l+7 of a chunk.  Per tile: light count, light and
 // heavy sums of q, heavy count, offset of the first heavy, and the offsets of
-// its heavies when it has at most 32 of them.
-template <int F32>
+// its heavies when it has at most kSparseOf(TILE) of them.
+template <int F32, int TILE>
 __device__ __forceinline__ void classify_body(const uint32_t *__restrict__ w, uint64_t n, int vec,
                                               const DevHeader *__restrict__ hdr, TileSum *__restrict__ agg,
                                               uint16_t *__restrict__ slist, uint32_t ntiles, uint32_t t_first,
                                               uint32_t t_stride)
 {
+    constexpr int kTile = TILE, kChunks = TILE / kChunk, kSparse = kSparseOf(TILE);
     __shared__ uint16_t s_list[kWarps][kSparse];
     if (block_stopped(hdr)) return;
     const uint32_t light_max = hdr->light_max;
@@ -577,12 +593,12 @@ __device__ __forceinline__ void classify_body(const uint32_t *__restrict__ w, ui
     }
 }
 
-template <int F32>
+template <int F32, int TILE>
 __global__ void __launch_bounds__(kThreads) k_classify(const uint32_t *__restrict__ w, uint64_t n, int vec,
                                                        const DevHeader *__restrict__ hdr, TileSum *__restrict__ agg,
                                                        uint16_t *__restrict__ slist, uint32_t ntiles)
 {
-    classify_body<F32>(w, n, vec, hdr, agg, slist, ntiles, blockIdx.x * kWarps + (threadIdx.x >> 5),
+    classify_body<F32, TILE>(w, n, vec, hdr, agg, slist, ntiles, blockIdx.x * kWarps + (threadIdx.x >> 5),
                        gridDim.x * kWarps);
 }
 
@@ -714,26 +730,25 @@ __global__ void __launch_bounds__(kThreads) k_tilescan(DevHeader *hdr, const Til
 }
 
 // ------------------------------------------------------------ k_split
-// For every tile c, from the tile prefix sums: with D_c = D at the first
-// light of tile c and E_c = E after the heavies before tile c,
-//   hb = max{ b : E(b) <= D_c }  -- the tile holding the first heavy item
-//        with E > D_c, the heavy current when tile c's first light is
-//        packed (the split of Alg. 3 on the heavy prefix sums);
-//   lb = max{ b : D(b) <= E_c }  -- a tile at or before the one holding the
-//        first light that follows tile c's first heavy (split on the light
-//        prefix sums);
+// For every tile boundary c = 0 .. ntiles, from the tile prefix sums: the
+// keys there (D: of the first light from tile c on, E: after the heavies
+// before tile c), the rank of the first heavy from tile c on, the tile's
+// heavies, and
+//   hb = max{ b : E(b) <= D(c) }  -- the tile holding the first heavy item
+//        with E > D(c), the heavy current when the first light from tile c
+//        on is packed (the split of Alg. 3 on the heavy prefix sums);
 //   next_heavy = position of the first heavy item after tile c.
 struct Prefix {
     uint64_t cl, ch;
     u128 L, H;
 };
 
-__device__ __forceinline__ Prefix prefix_at(const TileSum *incl, uint32_t b, uint64_t n)
+template <int TILE> __device__ __forceinline__ Prefix prefix_at(const TileSum *incl, uint32_t b, uint64_t n)
 {
     TileSum t = load_prefix(incl, b);
     Prefix p;
     p.cl = t.cl;
-    uint64_t end = (uint64_t)b * kTile;
+    uint64_t end = (uint64_t)b * TILE;
     if (end > n) end = n;
     p.ch = end - p.cl;
     p.L = mk128(t.l_lo, t.l_hi);
@@ -744,7 +759,8 @@ __device__ __forceinline__ Prefix prefix_at(const TileSum *incl, uint32_t b, uin
 __device__ __forceinline__ u128 key_E(const Prefix &p, uint64_t n, u128 Q) { return times_n(p.H, n) - (u128)p.ch * Q; }
 __device__ __forceinline__ u128 key_D(const Prefix &p, uint64_t n, u128 Q) { return (u128)p.cl * Q - times_n(p.L, n); }
 
-// Tile c of one table (one thread per tile).
+// Boundary c of one table (one thread per boundary).
+template <int TILE>
 __device__ __forceinline__ void split_body(const TileSum *__restrict__ incl, uint32_t ntiles, uint64_t n,
                                            DevHeader *hdr, Split *__restrict__ split, uint32_t c)
 {
@@ -752,470 +768,454 @@ __device__ __forceinline__ void split_body(const TileSum *__restrict__ incl, uin
     const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
     const uint64_t n_light = load_prefix(incl, ntiles).cl;
     if (c == 0) hdr->n_light = n_light;
-    if (c >= ntiles) return;
-    const Prefix pc = prefix_at(incl, c, n);
+    if (c > ntiles) return;
+    const Prefix pc = prefix_at<TILE>(incl, c, n);
     const u128 Dc = key_D(pc, n, Q), Ec = key_E(pc, n, Q);
     uint32_t lo = 0, hi = ntiles;
     while (lo < hi) {
         uint32_t mid = lo + (hi - lo + 1) / 2;
-        if (key_E(prefix_at(incl, mid, n), n, Q) <= Dc) lo = mid; else hi = mid - 1;
-    }
-    const uint32_t hb = lo;
-    lo = 0; hi = ntiles;
-    while (lo < hi) {
-        uint32_t mid = lo + (hi - lo + 1) / 2;
-        if (key_D(prefix_at(incl, mid, n), n, Q) <= Ec) lo = mid; else hi = mid - 1;
-    }
-    const uint32_t lb = lo;
-    const Prefix pn = prefix_at(incl, c + 1, n);
-    const uint64_t total_h = n - n_light;
-    uint32_t nxt = kNone;
-    if (pn.ch < total_h) { // heavy rank pn.ch is the first heavy of tile max{b : ch(b) <= pn.ch}
-        lo = c + 1; hi = ntiles - 1;
-        while (lo < hi) {
-            uint32_t mid = lo + (hi - lo + 1) / 2;
-            if (prefix_at(incl, mid, n).ch <= pn.ch) lo = mid; else hi = mid - 1;
-        }
-        const TileSum tb = tilesum_ldcg(incl + lo);
-        nxt = lo * (uint32_t)kTile + tb.first_heavy;
+        if (key_E(prefix_at<TILE>(incl, mid, n), n, Q) <= Dc) lo = mid; else hi = mid - 1;
     }
     Split s;
-    s.hb = hb; s.lb = lb; s.next_heavy = nxt; s.pad = 0;
-    split[c] = s;
+    s.hb = lo;
+    s.nheavy = 0;
+    s.next_heavy = kNone;
+    s.ch = (uint32_t)pc.ch;
+    s.d_lo = lo64(Dc); s.d_hi = hi64(Dc);
+    s.e_lo = lo64(Ec); s.e_hi = hi64(Ec);
+    if (c < ntiles) {
+        const Prefix pn = prefix_at<TILE>(incl, c + 1, n);
+        const uint64_t total_h = n - n_light;
+        s.nheavy = (uint32_t)(pn.ch - pc.ch);
+        if (pn.ch < total_h) { // heavy rank pn.ch is the first heavy of tile max{b : ch(b) <= pn.ch}
+            lo = c + 1; hi = ntiles - 1;
+            while (lo < hi) {
+                uint32_t mid = lo + (hi - lo + 1) / 2;
+                if (prefix_at<TILE>(incl, mid, n).ch <= pn.ch) lo = mid; else hi = mid - 1;
+            }
+            const TileSum tb = tilesum_ldcg(incl + lo);
+            s.next_heavy = lo * (uint32_t)TILE + tb.first_heavy;
+        }
+    }
+    const uint4 *src = reinterpret_cast<const uint4 *>(&s);
+    uint4 *dst = reinterpret_cast<uint4 *>(split + c);
+    dst[0] = src[0]; dst[1] = src[1]; dst[2] = src[2];
 }
 
+template <int TILE>
 __global__ void __launch_bounds__(kThreads) k_split(const TileSum *__restrict__ incl, uint32_t ntiles, uint64_t n,
                                                     DevHeader *hdr, Split *__restrict__ split)
 {
-    split_body(incl, ntiles, n, hdr, split, blockIdx.x * kThreads + threadIdx.x);
+    split_body<TILE>(incl, ntiles, n, hdr, split, blockIdx.x * kThreads + threadIdx.x);
 }
-
-
 
 // ------------------------------------------------------------ k_sweep
-// Tile c packs, as Alg. 3's pack does for one subproblem, the buckets of its
-// own lights and of every heavy item whose key E lies in (D_c, D_c'] (D_c:
-// key of the tile's first light, D_c': key after its last light): exactly
-// the items Alg. 2 packs while it consumes this tile's lights.  The heavy
-// items come tile by tile in index order from the tile k_split named
-// (Alg. 3's split on the heavy prefix sums); the first such tile is loaded
-// together with the own tile.  For each stream tile the block merges, in key
-// order, the own lights whose current heavy lies in that tile with the
-// tile's heavies in (D_c, D_c'] (heavy first when E <= D): a light step
-// takes the current heavy as its alias, a heavy step gets bucket
-// Q - (D_next - E) with D_next the key of the next light, and the next heavy
-// as alias.  The merged sequence is split evenly over the threads by a
-// merge-path co-rank search, then each thread walks its slice.
-__device__ __forceinline__ u128 nq_of(uint32_t x, uint32_t f32, int beta, uint32_t n32)
+// A task is a run of consecutive tiles c_first .. c_last - 1 (one subproblem
+// of Alg. 3): one warp packs the lights of these tiles and every heavy item
+// whose key E lies in (D(c_first), D(c_last)], exactly the items Alg. 2 packs
+// while it consumes these lights (wrs_pack.cuh).  The lights come from the
+// tiles themselves, 128 weights at a time; the heavies in index order from the
+// tile k_split named for the first of them, 128 weights at a time from a dense
+// tile or by the member lists of a run of sparse tiles (at most
+// kSparseOf(TILE) heavies each), until one lies past the task's last D.  While
+// the current heavy reaches past every light of the next 128-weight batches
+// (its key is that far ahead), the lights go straight from the loaded words to
+// their buckets: Zipf 1.5 has 2000 lights per heavy.
+//
+// Bound by instruction issue (n = 10^8 uniform: 10.2 warp instructions per
+// weight at 71 % issue; about 290 per batch of own weights, 320 per batch of
+// heavies' tile, 115 per search and 64 per 32 buckets stored).  It replaces a
+// block per eight tiles with 128-bit keys of a whole tile in shared memory, a
+// merge walked by threads and five barriers a tile.  n = 10^8, uniform / Zipf
+// 0.8 / Zipf 1.5: 1.54 / 1.50 / 1.18 -> 1.18 / 1.22 / 0.42 ms; n = 10^9 uniform
+// 15.4 -> 11.2 ms, Zipf 1.5 12.2 -> 3.3 ms.  One warp per block: the scheduler
+// replaces each warp as it ends, 19 -> 23 resident warps per SM (1.47 -> 1.40 ms
+// uniform).  The rings fit 24 warps per SM, the registers (80) too.
+__device__ __forceinline__ uint4 split_head(const Split *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
+template <typename K> __device__ __forceinline__ K split_D(const Split *p)
 {
-    if (!f32) return (u128)((uint64_t)x * n32);
-    const uint32_t ex = (x >> 23) & 0xFFu;
-    uint32_t m = x & 0x7FFFFFu;
-    if (ex) m |= 0x800000u;
-    const uint64_t nm = (uint64_t)m * n32; // < 2^56
-    const int sh = (ex ? (int)ex : 1) - 150 - beta;
-    return sh >= 0 ? ((u128)nm << sh) : (u128)(nm >> (-sh)); // exact: m carries the low zero bits
+    return kunpack<K>(__ldg(reinterpret_cast<const uint4 *>(p) + 1));
+}
+template <typename K> __device__ __forceinline__ K split_E(const Split *p)
+{
+    return kunpack<K>(__ldg(reinterpret_cast<const uint4 *>(p) + 2));
 }
 
-__device__ __forceinline__ u128 block_exclusive_scan1(u128 v, u128 &total, u128 *sm)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    u128 inc = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const u128 o = shfl_up128(inc, d);
-        if (lane >= d) inc += o;
-    }
-    if (lane == 31) sm[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        u128 t = lane < kWarps ? sm[lane] : (u128)0;
-#pragma unroll
-        for (int d = 1; d < kWarps; d <<= 1) {
-            const u128 o = shfl_up128(t, d);
-            if (lane >= d) t += o;
-        }
-        if (lane < kWarps) sm[lane] = t;
-    }
-    __syncthreads();
-    const u128 base = wid ? sm[wid - 1] : (u128)0;
-    total = sm[kWarps - 1];
-    __syncthreads();
-    return base + inc - v;
-}
+constexpr uint32_t kDirect = 128;        // weights a warp packs at once under one far heavy
+constexpr int kSweepTiles = 8;           // own tiles per task at most (the 32-bit keys cover 2^14 Q)
 
-// 16-B elements, 8 per 128-B bank row: XOR the column with the row's low bits
-// so that threads reading consecutive rows at one column hit distinct banks.
-__device__ __forceinline__ uint32_t swz(uint32_t j) { return j ^ ((j >> 3) & 7u); }
-
-struct SweepSmem {
-    u128 okey[kTile];     // keys D of the own lights, in order (swizzled)
-    u128 hkey[kTile];     // keys E of the current stream tile's heavies (swizzled)
-    uint16_t ooff[kTile];   // offsets of the own lights in the tile
-    uint16_t hoff[kTile];   // offsets of the stream tile's heavies
-    u128 scan[kWarps];
-    uint32_t cnt[kWarps];
-    uint32_t hcount;
-    uint32_t rng[4];      // light and heavy index ranges of the current round
-};
-
-// First index in [lo, hi) of the sorted keys whose key is > v (upper) or
-// >= v (!upper), found by a whole warp: each round probes 32 evenly spaced
-// keys and keeps the gap between the last probe before the answer and the
-// first one after it, so a range of 2048 takes two rounds and a final probe
-// of at most 32 keys.  Every lane returns the answer.
-__device__ __forceinline__ uint32_t warp_search(const u128 *key, uint32_t lo, uint32_t hi, u128 v, bool upper)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    while (hi - lo > 32) {
-        const uint32_t step = (hi - lo + 31) / 32;
-        const uint32_t p = lo + step * lane;
-        const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
-        const uint32_t cnt = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before)); // probes before the answer
-        if (cnt == 0) return lo;
-        const uint32_t nhi = lo + step * cnt; // first probe not before the answer (or past hi)
-        lo += step * (cnt - 1) + 1;
-        hi = nhi < hi ? nhi : hi;
-    }
-    const uint32_t p = lo + lane;
-    const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
-    return lo + (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before));
-}
-
-// Heavies of a stream tile up to which load_heavies compacts their words
-// first: the keys of heavies 0 .. c-1 end below byte 16 (c + 8) of the key
-// array, and the words sit in its top 4 c bytes (16 (c + 8) <= 32768 - 4 c).
-constexpr uint32_t kCompactMax = 1600;
-
-// Keys of stream tile t's heavies into S.hkey/S.hoff (all threads call).
-template <int F32>
-__device__ __forceinline__ void load_heavies(SweepSmem &S, uint32_t t, const uint32_t (&y)[kItems], uint32_t nheavy,
-                                             uint64_t n, uint32_t n32, const TileSum *incl,
-                                             const uint16_t *__restrict__ slist, const uint32_t *__restrict__ w,
-                                             u128 Q, uint32_t light_max, int beta)
-{
-    const Prefix pf = prefix_at(incl, t, n);
-    const u128 base = key_E(pf, n, Q);
-    const uint64_t tile0 = (uint64_t)t * kTile;
-    if (nheavy <= (uint32_t)kSparse) {
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-            u128 d = 0;
-            uint32_t off = 0;
-            if ((uint32_t)lane < nheavy) {
-                off = slist[(uint64_t)t * kSparse + lane];
-                d = nq_of(__ldg(w + tile0 + off), F32, beta, n32) - Q;
-            }
-            u128 key = d;
-#pragma unroll
-            for (int s = 1; s < 32; s <<= 1) {
-                const u128 o = shfl_up128(key, s);
-                if (lane >= s) key += o;
-            }
-            if ((uint32_t)lane < nheavy) { S.hkey[swz(lane)] = base + key; S.hoff[lane] = (uint16_t)off; }
-            if (lane == 0) S.hcount = nheavy;
-        }
-        __syncthreads();
-        return;
-    }
-    const uint64_t first = tile0 + (uint64_t)threadIdx.x * kItems;
-    uint32_t hm = 0;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k)
-        if (first + k < n && y[k] > light_max) hm |= 1u << k;
-    uint32_t ctot;
-    const uint32_t slot0 = block_exclusive_scan_u32((uint32_t)__popc(hm), ctot, S.cnt);
-    if (ctot <= kCompactMax) {
-        // Compacted first: the heavies' words go, in index order, to the top
-        // of the key array (below it the keys of the first ctot heavies
-        // never reach them), then thread t keys heavies [t q, t q + q),
-        // q = ceil(ctot / 256): every lane runs the same number of steps
-        // whatever the share of heavies in its eight words.
-        uint32_t *raw = reinterpret_cast<uint32_t *>(S.hkey) + (kTile * 4 - ctot);
-        {
-            uint32_t slot = slot0;
-#pragma unroll
-            for (int k = 0; k < kItems; ++k) {
-                if ((hm >> k) & 1u) {
-                    raw[slot] = y[k];
-                    S.hoff[slot] = (uint16_t)(threadIdx.x * kItems + k);
-                    ++slot;
-                }
-            }
-        }
-        __syncthreads();
-        const uint32_t q = (ctot + kThreads - 1) / kThreads;
-        const uint32_t j0 = min(threadIdx.x * q, ctot), j1 = min(j0 + q, ctot);
-        u128 sum = 0;
-        for (uint32_t j = j0; j < j1; ++j) {
-            const u128 e = nq_of(raw[j], F32, beta, n32) - Q;
-            S.hkey[swz(j)] = e;
-            sum += e;
-        }
-        u128 tot;
-        u128 key = base + block_exclusive_scan1(sum, tot, S.scan);
-        for (uint32_t j = j0; j < j1; ++j) {
-            key += S.hkey[swz(j)];
-            S.hkey[swz(j)] = key;
-        }
-        if (threadIdx.x == 0) S.hcount = ctot;
-        __syncthreads();
-        return;
-    }
-    // excesses n*q - Q into the key slots, then an in-place prefix
-    u128 sum = 0;
-    {
-        uint32_t slot = slot0;
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            if ((hm >> k) & 1u) {
-                const u128 e = nq_of(y[k], F32, beta, n32) - Q;
-                S.hkey[swz(slot)] = e;
-                S.hoff[slot] = (uint16_t)(threadIdx.x * kItems + k);
-                sum += e;
-                ++slot;
-            }
-        }
-    }
-    u128 tot;
-    u128 key = base + block_exclusive_scan1(sum, tot, S.scan);
-    {
-        const uint32_t cnt = (uint32_t)__popc(hm);
-        for (uint32_t j = 0; j < cnt; ++j) {
-            key += S.hkey[swz(slot0 + j)];
-            S.hkey[swz(slot0 + j)] = key;
-        }
-    }
-    if (threadIdx.x == 0) S.hcount = ctot;
-    __syncthreads();
-}
-
-constexpr int kSweepTiles = 8; // own tiles per block of k_sweep (they share stream tiles)
-
-// Own tiles [c_first, c_last) of one table.
-template <int F32>
-__device__ __forceinline__ void sweep_body(const uint32_t *__restrict__ w, uint64_t n, int vec, DevHeader *hdr,
-                                           const TileSum *__restrict__ incl, const Split *__restrict__ split,
+template <int F32, int MODE, int TILE>
+__device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *__restrict__ w, uint64_t n, int vec,
+                                           DevHeader *hdr, const Split *__restrict__ split,
                                            const uint16_t *__restrict__ slist, uint32_t ntiles,
-                                           uint4 *__restrict__ table, uint32_t c_first, uint32_t c_last,
-                                           bool force_wide = false)
+                                           uint4 *__restrict__ table, uint32_t c_first, uint32_t c_last, u128 Q)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    SweepSmem &S = *reinterpret_cast<SweepSmem *>(smem_raw);
-    if (block_stopped(hdr)) return;
-    const uint32_t n32 = (uint32_t)n;
-    const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
+    using K = typename Units<F32, MODE>::K;
+    constexpr bool kWide = MODE == kPackQ128;
+    constexpr int kTile = TILE, kSparse = kSparseOf(TILE);
+    constexpr int kPer = WarpRings<MODE>::kPer;
+    constexpr uint32_t kBatch = WarpRings<MODE>::kBatch, kRing = WarpRings<MODE>::kRing;
+    const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const uint32_t light_max = hdr->light_max;
-    const int beta = hdr->beta;
-    const uint32_t shift = hdr->shift;
-    const bool narrow = shift == 0 && !force_wide; // Q < 2^64, the same for the whole grid
+    Units<F32, MODE> U;
+    U.init(Q, n, hdr->beta, hdr->shift);
     bool bad = false;
 
-    uint32_t x[kItems], y[kItems];
-    load_items(w, n, vec, (uint64_t)c_first * kTile + (uint64_t)threadIdx.x * kItems, x);
-    uint32_t s = split[c_first].hb;   // current stream tile
-    uint32_t s_loaded = kNone;        // stream tile whose heavies are in S.hkey
-    uint32_t y_tile = kNone;          // stream tile whose words are in y
-    if (s < ntiles) { load_items(w, n, vec, (uint64_t)s * kTile + (uint64_t)threadIdx.x * kItems, y); y_tile = s; }
-
-    for (uint32_t c = c_first; c < c_last; ++c) {
-        const uint64_t tile0 = (uint64_t)c * kTile;
-        const uint64_t first = tile0 + (uint64_t)threadIdx.x * kItems;
-        // own lights: deficits Q - n*q, thresholds n*q >> shift, full lights
-        uint32_t lmask = 0;
-#pragma unroll
-        for (int k = 0; k < kItems; ++k)
-            if (first + k < n && x[k] <= light_max) lmask |= 1u << k;
-        uint32_t nl;
-        const uint32_t lslot0 = block_exclusive_scan_u32((uint32_t)__popc(lmask), nl, S.cnt); // syncs: okey free
-        u128 def = 0;
-        {
-            uint32_t slot = lslot0;
-#pragma unroll
-            for (int k = 0; k < kItems; ++k) {
-                if ((lmask >> k) & 1u) {
-                    const u128 d = Q - nq_of(x[k], F32, beta, n32);
-                    S.okey[swz(slot)] = d;
-                    S.ooff[slot] = (uint16_t)(threadIdx.x * kItems + k);
-                    def += d;
-                    ++slot;
-                }
-            }
-        }
-        const Prefix pc = prefix_at(incl, c, n);
-        const u128 D_start = key_D(pc, n, Q);
-        u128 dtot;
-        {
-            u128 kl = D_start + block_exclusive_scan1(def, dtot, S.scan);
-            const uint32_t cnt = (uint32_t)__popc(lmask);
-            for (uint32_t j = 0; j < cnt; ++j) { // deficits -> exclusive keys, in place
-                const u128 d = S.okey[swz(lslot0 + j)];
-                S.okey[swz(lslot0 + j)] = kl;
-                kl += d;
-            }
-        }
-        const u128 D_end = D_start + dtot;
-        // prefetch the next own tile
-        if (c + 1 < c_last) load_items(w, n, vec, (uint64_t)(c + 1) * kTile + (uint64_t)threadIdx.x * kItems, x);
-        if (nl == 0) continue; // no lights: nothing is packed for this tile
-        uint32_t al = 0; // own lights resolved so far
-        for (;;) {
-            if (s >= ntiles) {
-                // no heavy item left: the remaining own lights must be exactly full
-                __syncthreads();
-                for (uint32_t i = al + threadIdx.x; i < nl; i += kThreads) {
-                    const u128 dn = (i + 1 < nl) ? S.okey[swz(i + 1)] : D_end;
-                    const u128 nq = Q - (dn - S.okey[swz(i)]);
-                    if (nq != Q) bad = true;
-                    const uint32_t me = (uint32_t)(tile0 + S.ooff[i]);
-                    put_bucket(table, me, lo64(nq >> shift), me, n, hdr);
-                }
-                break;
-            }
-            if (s != s_loaded) {
-                const uint32_t nheavy = tilesum_ldcg(incl + s).nheavy;
-                if (nheavy == 0) { // on to the tile of the first heavy after this one
-                    const uint32_t nh = split[s].next_heavy;
-                    s = nh == kNone ? ntiles : nh / (uint32_t)kTile;
-                    continue;
-                }
-                if (y_tile != s && nheavy > (uint32_t)kSparse) {
-                    load_items(w, n, vec, (uint64_t)s * kTile + (uint64_t)threadIdx.x * kItems, y);
-                    y_tile = s;
-                }
-                __syncthreads(); // previous window consumed
-                load_heavies<F32>(S, s, y, nheavy, n, n32, incl, slist, w, Q, light_max, beta);
-                s_loaded = s;
-                if (s + 1 < ntiles) { // prefetch the following stream tile
-                    load_items(w, n, vec, (uint64_t)(s + 1) * kTile + (uint64_t)threadIdx.x * kItems, y);
-                    y_tile = s + 1;
-                }
-            }
-            const uint32_t hc = S.hcount;
-            // position of the first heavy after stream tile s (kNone: none),
-            // read while the block waits at the barrier
-            const uint32_t hnext = split[s].next_heavy;
-            __syncthreads(); // own keys and window complete
-            if (threadIdx.x < 3 * 32) { // one warp per search
-                const int q = threadIdx.x >> 5;
-                uint32_t r;
-                if (q == 0) r = warp_search(S.okey, al, nl, S.hkey[swz(hc - 1)], false); // lights answered here
-                else if (q == 1) r = warp_search(S.hkey, 0, hc, D_start, true);          // heavies packed here:
-                else r = warp_search(S.hkey, 0, hc, D_end, true);                        // E in (D_start, D_end]
-                if ((threadIdx.x & 31) == 0) S.rng[1 + q] = r;
-            }
-            __syncthreads();
-            const uint32_t a0 = al, a1 = S.rng[1], b0 = S.rng[2], b1 = S.rng[3];
-            if (WRS_CHECK && !check_ok(hc <= (uint32_t)kTile && nl <= (uint32_t)kTile && a0 <= a1 && a1 <= nl &&
-                                           b0 <= b1 && b1 <= hc, hdr))
-                break;
-            const uint32_t na = a1 - a0, nb = b1 > b0 ? b1 - b0 : 0, M = na + nb;
-            const uint32_t per = (M + kThreads - 1) / kThreads;
-            const uint64_t sbase = (uint64_t)s * kTile;
-            const uint32_t d0 = threadIdx.x * per;
-            if (d0 < M) {
-                // co-rank: number of heavies among the first d0 merged elements
-                uint32_t lo = d0 > na ? d0 - na : 0, hi = d0 < nb ? d0 : nb;
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi + 1) >> 1; // is heavy b0+mid-1 before light a0+d0-mid?
-                    if (S.hkey[swz(b0 + mid - 1)] <= S.okey[swz(a0 + d0 - mid)]) lo = mid; else hi = mid - 1;
-                }
-                uint32_t j = b0 + lo, i = a0 + (d0 - lo);
-                const uint32_t steps = min(per, M - d0);
-                u128 ej = j < b1 ? S.hkey[swz(j)] : (u128)0;
-                u128 di = i < nl ? S.okey[swz(i)] : D_end; // key of light i (D_end past the last)
-                // positions of heavies j and j + 1 (the first heavy after the
-                // stream tile past its last), kept in registers along the walk
-                auto hpos = [&](uint32_t jj) -> uint32_t {
-                    return jj < hc ? (uint32_t)(sbase + S.hoff[jj]) : hnext;
-                };
-                uint32_t hp = hpos(j), hp1 = hpos(j + 1);
-                if (narrow) {
-                    // Q < 2^64 (shift 0): a bucket's mass, a light's deficit
-                    // and a heavy's gap D - E (< Q when the build is sound,
-                    // checked in full) are 64-bit; only the keys are wider
-                    const uint64_t Q64 = lo64(Q);
-                    for (uint32_t st = 0; st < steps; ++st) {
-                        const bool heavy_next = (j < b1) && (i >= a1 || ej <= di);
-                        uint32_t me, alias;
-                        uint64_t bw;
-                        if (heavy_next) {
-                            const u128 gap = di - ej;
-                            if (hi64(gap) != 0 || lo64(gap) >= Q64) bad = true;
-                            bw = Q64 - lo64(gap);
-                            me = hp;
-                            if (hp1 == kNone && bw != Q64) bad = true;
-                            alias = (hp1 == kNone || bw == Q64) ? me : hp1;
-                            ++j;
-                            if (j < b1) ej = S.hkey[swz(j)];
-                            hp = hp1;
-                            hp1 = hpos(j + 1);
-                        } else {
-                            if (WRS_CHECK && !check_ok(i < a1, hdr)) break;
-                            const u128 dn = (i + 1 < nl) ? S.okey[swz(i + 1)] : D_end;
-                            const uint64_t def = lo64(dn) - lo64(di); // < Q: exact modulo 2^64
-                            bw = Q64 - def;
-                            me = (uint32_t)(tile0 + S.ooff[i]);
-                            alias = (def == 0) ? me : hp;
-                            ++i;
-                            di = dn;
-                        }
-                        put_bucket(table, me, bw, alias, n, hdr);
-                    }
-                } else {
-                    for (uint32_t st = 0; st < steps; ++st) {
-                        const bool heavy_next = (j < b1) && (i >= a1 || ej <= di);
-                        uint32_t me, alias;
-                        u128 bw;
-                        if (heavy_next) {
-                            const u128 gap = di - ej;
-                            if (gap >= Q) bad = true;
-                            bw = Q - gap;
-                            me = hp;
-                            if (hp1 == kNone && bw != Q) bad = true;
-                            alias = (hp1 == kNone || bw == Q) ? me : hp1;
-                            ++j;
-                            if (j < b1) ej = S.hkey[swz(j)];
-                            hp = hp1;
-                            hp1 = hpos(j + 1);
-                        } else { // light i; j < hc: heavy j is its current heavy
-                            if (WRS_CHECK && !check_ok(i < a1, hdr)) break;
-                            const u128 dn = (i + 1 < nl) ? S.okey[swz(i + 1)] : D_end;
-                            bw = Q - (dn - di);
-                            me = (uint32_t)(tile0 + S.ooff[i]);
-                            alias = (bw == Q) ? me : hp;
-                            ++i;
-                            di = dn;
-                        }
-                        put_bucket(table, me, lo64(bw >> shift), alias, n, hdr);
-                    }
-                }
-            }
-            al = a1;
-            if (b1 < hc) { // the first heavy past D_end is in this tile: this own tile is done
-                // end of the subproblem: the stream tile carried to the next
-                // own tile is the one k_split found for it independently
-                if (WRS_CHECK && threadIdx.x == 0 && c + 1 < ntiles) check_ok(split[c + 1].hb == s, hdr);
-                break;
-            }
-            s = hnext == kNone ? ntiles : hnext / (uint32_t)kTile; // the next stream tile with a heavy
-        }
+    // lights: ranks [li, lh) are in the ring, weights from `at` on are not read yet (x: the next batch)
+    uint64_t at = (uint64_t)c_first * kTile;
+    const uint64_t end = min((uint64_t)c_last * kTile, n);
+    uint32_t li = 0, lh = 0, x[kPer];
+    load_lane(w, vec, at, end, 0xFFFFFFFFu, x);
+    const K d_base = split_D<K>(split + c_first);
+    const KeyFrame<K> f = key_frame(ksub(split_D<K>(split + c_last), d_base));
+    K drun{0, 0}; // D of light lh
+    // heavies: ranks [hj, hh) are in the ring; the next come from weight sa of tile s on (y: the next batch)
+    uint32_t s = split_head(split + c_first).x;
+    uint32_t hj = 0, hh = 0, y[kPer];
+    uint4 rs = make_uint4(0, 0, 0, 0);
+    uint64_t sa = 0, send = 0;
+    bool past = false;  // the last heavy in the ring lies past the task's last D
+    K erun{0, 0};       // E of heavy hh - 1
+    if (s < ntiles) {
+        rs = split_head(split + s);
+        erun = ksub(split_E<K>(split + s), d_base);
+        sa = (uint64_t)s * kTile;
+        send = min(sa + kTile, n);
+        if (rs.z > (uint32_t)kSparse) load_lane(w, vec, sa, send, 0u, y);
     }
+    if (lane == 0) R.kp[R.heavy(0)].y = kNone;
+
+    // 128 Q in units of the 32-bit keys, rounded up: the most a batch of lights can add to D
+    const uint32_t batch_units = min(kshr32(kmul(U.Q, kDirect), f.s) + 2u, 1u << 30);
+    const bool far_batches = kbits(kmul(U.Q, kDirect)) < f.s + 30;
+    if (lane == 0) R.put(R.light(0), drun, 0u, kNone);
+
+    for (;;) {
+        if (lh - li < 32 && at < end && (hh != hj || s >= ntiles)) { // the next own weights
+            // Direct: the current heavy reaches past every light of the next
+            // batches, so these lights go straight from the weights to their buckets.
+            const uint32_t klast = R.kp[R.light(lh)].x; // of D[lh]
+            const uint32_t kfirst = hh == hj ? 0u : R.kp[R.heavy(hj)].x;
+            uint32_t batches = 0;
+            if (far_batches && (int32_t)kfirst > 0) {
+                if (kfirst == 0x7FFFFFFFu) batches = 1u << 20;
+                else if (kfirst > klast + batch_units) batches = (kfirst - klast - 1) / batch_units;
+            }
+            if (batches >= 2 && li == lh) {
+                const uint32_t hp = R.kp[R.heavy(hj)].y;
+                K sum{0, 0};
+                K96 Ql;
+                Ql.lo = U.Q.lo;
+                Ql.hi = (uint32_t)U.Q.hi;
+                uint32_t z[4], c = 0;
+                const uint64_t left = (end - at + kDirect - 1) / kDirect;
+                if (batches > left) batches = (uint32_t)left;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) z[k] = at + 32 * k + lane < end ? __ldg(w + at + 32 * k + lane) : 0xFFFFFFFFu;
+                for (;;) {
+                    uint32_t zn[4];
+                    const uint64_t an = at + kDirect;
+                    const bool more = c + 1 < batches;
+                    if (more) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) zn[k] = an + 32 * k + lane < end ? __ldg(w + an + 32 * k + lane) : 0xFFFFFFFFu;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (z[k] <= light_max) {
+                            const K96 nq = U.nq_light(z[k]);
+                            const K96 df = ksub(Ql, nq);
+                            sum = kadd96(sum, df);
+                            const uint32_t me = (uint32_t)at + 32 * k + lane;
+                            K bw;
+                            bw.lo = nq.lo;
+                            bw.hi = nq.hi;
+                            put_bucket(table, me, U.thr(bw), kzero(df) ? me : hp, n, hdr);
+                        }
+                    }
+                    at = an;
+                    ++c;
+                    if (!more) break;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) z[k] = zn[k];
+                }
+                if (at < end) load_lane(w, vec, at, end, 0xFFFFFFFFu, x);
+                drun = kadd(drun, kshfl(warp_scan_key(sum), 31));
+                lh += kRing; // the same entry; ranks only have to differ from the task's first light's, 0
+                li = lh;
+                if (lane == 0) R.put(R.light(lh), drun, key32_light(f, drun), kNone);
+                __syncwarp();
+                continue;
+            }
+            if (batches < 2) {
+                uint32_t m = 0;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k)
+                    if (x[k] <= light_max) m |= 1u << k; // past the end: never light
+                Light<MODE> v[kPer];
+                K sum{0, 0};
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    v[k].set(U, x[k], (m >> k) & 1u);
+                    sum = v[k].add(sum);
+                }
+                const uint32_t pos = (uint32_t)at + kPer * lane;
+                at += kBatch;
+                if (at < end) load_lane(w, vec, at, end, 0xFFFFFFFFu, x);
+                sum = kput(sum, (uint32_t)__popc(m));
+                const K exc = ksub(warp_scan_key(sum), sum);
+                K run = kadd(drun, kvalue(exc));
+                uint32_t r = lh + kcount(exc);
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    if ((m >> k) & 1u) {
+                        const uint32_t e = R.light(r);
+                        R.put(e, run, key32_light(f, run), pos + k);
+                        ++r;
+                    }
+                    run = v[k].add(run);
+                }
+                if (lane == 31) R.put(R.light(r), run, key32_light(f, run), kNone); // the entry after the last light
+                drun = kshfl(run, 31);
+                lh = __shfl_sync(0xFFFFFFFFu, r, 31);
+                __syncwarp();
+                continue;
+            }
+        }
+        if (hh - hj < 33 && !past && s < ntiles) { // the next batch of heavies (the last one's alias is the one after it)
+            uint32_t tot;
+            if (rs.z > (uint32_t)kSparse) {
+                uint32_t m = 0;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k)
+                    if (y[k] > light_max) m |= 1u << k; // past the end: never heavy
+                uint32_t r = 0;
+                if (MODE != kPackQ32) r = hh + warp_rank<kPer>(m, tot); // the sums may need their top bits
+                Heavy<MODE> v[kPer];
+                K sum{0, 0};
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    v[k].set(U, y[k], (m >> k) & 1u);
+                    sum = v[k].add(sum);
+                }
+                const uint32_t pos = (uint32_t)sa + kPer * lane;
+                sa += kBatch;
+                bool next_tile = false;
+                if (sa < send) load_lane(w, vec, sa, send, 0u, y);
+                else next_tile = true;
+                if (MODE == kPackQ32) sum = kput(sum, (uint32_t)__popc(m));
+                const K inc = warp_scan_key(sum);
+                K exc = ksub(inc, sum);
+                if (MODE == kPackQ32) {
+                    r = hh + kcount(exc);
+                    exc = kvalue(exc);
+                }
+                K run = kadd(erun, exc);
+                bool skip = false; // every heavy of the batch comes before the task's first light
+                if (hh == 0) {
+                    K after = run;
+#pragma unroll
+                    for (int k = 0; k < kPer; ++k) after = v[k].add(after);
+                    after = kshfl(after, 31);
+                    skip = kneg(after) || kzero(after);
+                    if (skip) erun = after;
+                }
+                if (!skip) {
+#pragma unroll
+                    for (int k = 0; k < kPer; ++k) {
+                        if ((m >> k) & 1u) {
+                            run = v[k].add(run);
+                            const uint32_t e = R.heavy(r);
+                            R.put(e, run, key32_heavy(f, run), pos + k);
+                            ++r;
+                        }
+                    }
+                    erun = kshfl(run, 31);
+                    hh = __shfl_sync(0xFFFFFFFFu, r, 31);
+                }
+                if (next_tile) {
+                    s = rs.y == kNone ? ntiles : rs.y / (uint32_t)kTile;
+                    if (s < ntiles) {
+                        rs = split_head(split + s);
+                        sa = (uint64_t)s * kTile;
+                        send = min(sa + kTile, n);
+                        if (rs.z > (uint32_t)kSparse) load_lane(w, vec, sa, send, 0u, y);
+                    }
+                }
+            } else {
+                // sparse tiles s .. s + 31 up to the first dense one, while their heavies fit a batch
+                const uint32_t t = s + lane;
+                uint4 rt = make_uint4(0, 0, 0, 0);
+                bool ok = t < ntiles && t >= s;
+                if (ok) rt = split_head(split + t);
+                ok = ok && rt.z <= (uint32_t)kSparse;
+                uint32_t inc = ok ? rt.z : kRing; // a refused tile ends the run
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                    if (lane >= (uint32_t)d) inc += o;
+                }
+                const uint32_t took = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, inc <= kBatch)); // a prefix, not empty
+                tot = __shfl_sync(0xFFFFFFFFu, inc, took - 1);
+                const uint32_t next = __shfl_sync(0xFFFFFFFFu, rt.y, took - 1);
+                __syncwarp();
+                if (lane < took) {
+                    const uint32_t r0 = hh + inc - rt.z;
+                    for (uint32_t q = 0; q < rt.z; ++q) {
+                        const uint32_t pos = t * (uint32_t)kTile + slist[(uint64_t)t * kSparse + q];
+                        const uint32_t e = R.heavy(r0 + q);
+                        R.kp[e] = make_uint2(__ldg(w + pos), pos);
+                    }
+                }
+                __syncwarp();
+                for (uint32_t r0 = 0; r0 < tot; r0 += 32) { // words -> keys, 32 at a time
+                    const uint32_t e = R.heavy(hh + r0 + lane);
+                    const bool in = r0 + lane < tot;
+                    const K v = in ? ksub(U.nq(R.kp[e].x), U.Q) : K{0, 0};
+                    const K run = kadd(erun, warp_scan_key(v));
+                    if (in) R.put(e, run, key32_heavy(f, run), R.kp[e].y);
+                    erun = kshfl(run, 31);
+                }
+                hh += tot;
+                s = next == kNone ? ntiles : next / (uint32_t)kTile;
+                if (s < ntiles) {
+                    rs = split_head(split + s);
+                    sa = (uint64_t)s * kTile;
+                    send = min(sa + kTile, n);
+                    if (rs.z > (uint32_t)kSparse) load_lane(w, vec, sa, send, 0u, y);
+                }
+            }
+            past = !kle(erun, f.dmax) && hh != hj;
+            if (s >= ntiles && lane == 0) R.kp[R.heavy(hh)].y = kNone; // no heavy after the last
+            __syncwarp();
+            continue;
+        }
+        // Merge the next outputs, up to 63: those that the next 31 lights, D
+        // of the one after them and the next 32 heavies decide.
+        const uint32_t na = min(31u, lh - li), nb = hh - hj;
+        const uint32_t kd = R.kp[R.light(li + lane)].x;
+        uint32_t ke = R.kp[R.heavy(hj + lane)].x;
+        if (lane >= nb) ke = 0x7FFFFFFFu;
+        uint32_t cnt = 0; // heavies before light `lane` among the 32
+        if ((int32_t)__shfl_sync(0xFFFFFFFFu, ke, 0) <= (int32_t)__shfl_sync(0xFFFFFFFFu, kd, na)) {
+#pragma unroll
+            for (uint32_t st = 16; st; st >>= 1) {
+                const uint32_t v = __shfl_sync(0xFFFFFFFFu, ke, cnt + (st - 1));
+                if ((int32_t)v <= (int32_t)kd) cnt += st;
+            }
+            if ((int32_t)__shfl_sync(0xFFFFFFFFu, ke, cnt) <= (int32_t)kd) ++cnt;
+            if (f.s != 0) {
+                const uint32_t last = __shfl_sync(0xFFFFFFFFu, ke, cnt - 1);
+                if (__any_sync(0xFFFFFFFFu, last == kd && cnt > 0 && lane <= na)) { // rare: told apart by the exact keys
+                    while (cnt > 0 && lane <= na) {
+                        const uint32_t eh = R.heavy(hj + cnt - 1), el = R.light(li + lane);
+                        if (R.kp[eh].x != kd) break;
+                        const uint64_t a = R.low[el], b = R.low[eh];
+                        if (kWide ? (int32_t)(R.high[el] - R.high[eh] - (a < b ? 1u : 0u)) >= 0 : (int64_t)(a - b) >= 0) break;
+                        --cnt;
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+        // merged position of light `lane`; the outputs end where light na
+        // would come, or after the 32nd heavy
+        const uint32_t p = lane + cnt;
+        uint32_t total = __shfl_sync(0xFFFFFFFFu, p, na);
+        if (total == 0) break;
+        if (total == na + 32) total = 32 + (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, cnt < 32 && lane < na));
+        if (total > 32 && total < 48) total = 32; // a second pass for few outputs does not pay
+        const bool now = lane < na && p < total;
+        uint32_t lights = __reduce_or_sync(0xFFFFFFFFu, now ? shl32(1u, p) : 0u);
+        const uint32_t lights2 = total > 32 ? __reduce_or_sync(0xFFFFFFFFu, now ? shl32(1u, p - 32u) : 0u) : 0u;
+        for (;;) { // outputs 0 .. 31, then 32 .. 62
+            const bool is_light = (lights >> lane) & 1u;
+            const uint32_t a = (uint32_t)__popc(lights & lt), b = lane - a; // lights and heavies before it (of its pass)
+            if (lane < total) {
+                // light: Q - (D[a + 1] - D[a]), alias heavy b; heavy: Q + E[b] - D[a], alias heavy b + 1
+                const uint32_t ea = R.light(li + a), eb = R.heavy(hj + b);
+                const uint32_t eo = is_light ? R.light(li + a + 1) : eb, et = is_light ? ea : R.heavy(hj + b + 1);
+                const uint32_t hp = R.kp[eb].y, ot = R.kp[et].y;
+                const uint32_t me = is_light ? ot : hp;
+                uint32_t alias = is_light ? hp : ot;
+                const uint64_t dl = R.low[ea], ol = R.low[eo];
+                bool wrong;
+                uint64_t thr;
+                if (!kWide) { // exact modulo 2^64: 0 <= bucket <= Q < 2^64
+                    const uint64_t df = ol - dl, flip = is_light ? ~0ull : 0ull;
+                    const uint64_t bw = U.Q.lo + (df ^ flip) + (is_light ? 1u : 0u);
+                    if (bw == U.Q.lo) alias = me;
+                    wrong = bw > U.Q.lo;
+                    thr = bw;
+                } else {      // modulo 2^96
+                    K da, od;
+                    da.lo = dl;
+                    da.hi = R.high[ea];
+                    od.lo = ol;
+                    od.hi = R.high[eo];
+                    K bw = kadd(U.Q, is_light ? ksub(da, od) : ksub(od, da));
+                    bw.hi &= 0xFFFFFFFFu;
+                    if (keq(bw, U.Q)) alias = me;
+                    wrong = !kle(bw, U.Q);
+                    thr = U.thr(bw);
+                }
+                // heavies before the task's first light belong to the task before
+                if (is_light || li + a != 0) {
+                    if (alias == kNone || wrong) bad = true; // a part-filled last heavy; D - E >= Q
+                    else put_bucket(table, me, thr, alias, n, hdr);
+                }
+            }
+            const uint32_t outs = min(total, 32u), took = (uint32_t)__popc(lights);
+            li += took;
+            hj += outs - took;
+            total -= outs;
+            if (total == 0) break;
+            lights = lights2;
+        }
+        __syncwarp(); // entries read before they are replaced
+    }
+    if (!kzero(ksub(drun, f.dmax))) bad = true;
+    // end of the subproblem: the heavy carried on lies in the tile k_split
+    // found independently
+    if (WRS_CHECK && lane == 0 && hj < hh)
+        check_ok(R.kp[R.heavy(hj)].y / (uint32_t)kTile == split_head(split + c_last).x, hdr);
+    return bad;
+}
+
+// Task (c_first, c_last) of one table for this warp.
+template <int F32, int TILE>
+__device__ __forceinline__ void sweep_body(const uint32_t *__restrict__ w, uint64_t n, int vec, DevHeader *hdr,
+                                           const Split *__restrict__ split, const uint16_t *__restrict__ slist,
+                                           uint32_t ntiles, uint4 *__restrict__ table, uint32_t c_first,
+                                           uint32_t c_last, bool force_wide = false)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (__shfl_sync(0xFFFFFFFFu, *(volatile const uint32_t *)&hdr->status, 0)) return; // the whole warp or none
+    const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
+    const uint32_t mode = force_wide ? (uint32_t)kPackQ128 : hdr->f32 >> 8; // the same for the whole grid
+    bool bad;
+    if (mode == kPackQ32)
+        bad = sweep_task<F32, kPackQ32, TILE>(*reinterpret_cast<WarpRings<kPackQ32> *>(smem_raw), w, n, vec, hdr, split,
+                                        slist, ntiles, table, c_first, c_last, Q);
+    else if (F32 && mode == kPackQ96)
+        bad = sweep_task<F32, kPackQ96, TILE>(*reinterpret_cast<WarpRings<kPackQ96> *>(smem_raw), w, n, vec, hdr, split,
+                                        slist, ntiles, table, c_first, c_last, Q);
+    else
+        bad = sweep_task<F32, kPackQ128, TILE>(*reinterpret_cast<WarpRings<kPackQ128> *>(smem_raw), w, n, vec, hdr,
+                                         split, slist, ntiles, table, c_first, c_last, Q);
     if (bad) set_status(hdr, kEInternal);
 }
 
-// Block b packs own tiles [b * group, (b + 1) * group): one subproblem of
-// Alg. 3 per block (group = kSweepTiles unless the caller asks for a split
-// count); force_wide runs the 128-bit walk even when Q < 2^64.
-template <int F32>
-__global__ void __launch_bounds__(kThreads, 3) k_sweep(const uint32_t *__restrict__ w, uint64_t n, int vec,
-                                                       DevHeader *hdr, const TileSum *__restrict__ incl,
-                                                       const Split *__restrict__ split,
-                                                       const uint16_t *__restrict__ slist, uint32_t ntiles,
-                                                       uint4 *__restrict__ table, uint32_t group, int force_wide)
+// Block (warp) v packs own tiles [v * group, (v + 1) * group); force_wide runs
+// the 128-bit keys even when 96 bits hold them.
+template <int F32, int TILE>
+__global__ void __launch_bounds__(32, kPackBlocks) k_sweep(const uint32_t *__restrict__ w, uint64_t n, int vec,
+                                                              DevHeader *hdr, const Split *__restrict__ split,
+                                                              const uint16_t *__restrict__ slist, uint32_t ntiles,
+                                                              uint4 *__restrict__ table, uint32_t group, int force_wide)
 {
     const uint32_t c_first = blockIdx.x * group;
-    sweep_body<F32>(w, n, vec, hdr, incl, split, slist, ntiles, table, c_first, min(c_first + group, ntiles),
+    sweep_body<F32, TILE>(w, n, vec, hdr, split, slist, ntiles, table, c_first, min(c_first + group, ntiles),
                     force_wide != 0);
 }
 

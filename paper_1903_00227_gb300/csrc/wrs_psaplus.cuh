@@ -27,6 +27,44 @@
 
 namespace wrs {
 
+__device__ __forceinline__ u128 nq_of(uint32_t x, uint32_t f32, int beta, uint32_t n32)
+{
+    if (!f32) return (u128)((uint64_t)x * n32);
+    const uint32_t ex = (x >> 23) & 0xFFu;
+    uint32_t m = x & 0x7FFFFFu;
+    if (ex) m |= 0x800000u;
+    const uint64_t nm = (uint64_t)m * n32; // < 2^56
+    const int sh = (ex ? (int)ex : 1) - 150 - beta;
+    return sh >= 0 ? ((u128)nm << sh) : (u128)(nm >> (-sh)); // exact: m carries the low zero bits
+}
+
+// 16-B elements, 8 per 128-B bank row: XOR the column with the row's low bits
+// so that threads reading consecutive rows at one column hit distinct banks.
+__device__ __forceinline__ uint32_t swz(uint32_t j) { return j ^ ((j >> 3) & 7u); }
+
+// First index in [lo, hi) of the sorted keys whose key is > v (upper) or
+// >= v (!upper), found by a whole warp: each round probes 32 evenly spaced
+// keys and keeps the gap between the last probe before the answer and the
+// first one after it, so a range of 2048 takes two rounds and a final probe
+// of at most 32 keys.  Every lane returns the answer.
+__device__ __forceinline__ uint32_t warp_search(const u128 *key, uint32_t lo, uint32_t hi, u128 v, bool upper)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    while (hi - lo > 32) {
+        const uint32_t step = (hi - lo + 31) / 32;
+        const uint32_t p = lo + step * lane;
+        const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
+        const uint32_t cnt = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before)); // probes before the answer
+        if (cnt == 0) return lo;
+        const uint32_t nhi = lo + step * cnt; // first probe not before the answer (or past hi)
+        lo += step * (cnt - 1) + 1;
+        hi = nhi < hi ? nhi : hi;
+    }
+    const uint32_t p = lo + lane;
+    const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
+    return lo + (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before));
+}
+
 // Leftover sums of tiles: l = deficits of the lights (v <= Q), h = excesses
 // of the heavies, cl / nheavy = their counts (TileSum's fields).
 __device__ __forceinline__ void pp_add(TileSum &a, const TileSum &b)
