@@ -155,6 +155,11 @@ uint32_t sweep_group(uint32_t ntiles, uint32_t most)
     return g;
 }
 
+// Tables of at most kTile weights in one launch (wrs_batch.cuh).
+wrs_status small_attributes();
+void launch_small(cudaStream_t s, bool f32, const uint32_t *w, uint64_t n, int vec, DevHeader *hdr, uint4 *buckets,
+                  int acc);
+
 std::atomic<bool> g_attr_done[64];
 std::mutex g_attr_mu;
 
@@ -169,7 +174,7 @@ wrs_status set_kernel_attributes()
     cudaError_t e = cudaSuccess;
     for (auto *k : {k_sweep<0, kTile>, k_sweep<1, kTile>, k_sweep<0, kFineTile>, k_sweep<1, kFineTile>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return WRS_EDEVICE;
+    if (e != cudaSuccess || small_attributes() != WRS_OK) return WRS_EDEVICE;
     g_attr_done[dev].store(true, std::memory_order_release);
     return WRS_OK;
 }
@@ -315,22 +320,28 @@ wrs_status enqueue_build(wrs_table *t, const void *d_weights, uint64_t n, wrs_dt
     }
     const bool tm = t->timing != 0;
     if (tm) cudaEventRecord(t->ev[0], s);
-    if (f32) k_stats<1><<<nparts, kThreads, 0, s>>>(w, n, vec, t->part);
-    else k_stats<0><<<nparts, kThreads, 0, s>>>(w, n, vec, t->part);
-    if (tm) cudaEventRecord(t->ev[1], s);
-    k_stats_combine<<<1, kThreads, 0, s>>>(t->part, nparts, n, f32, t->hdr);
-    if (tm) cudaEventRecord(t->ev[2], s);
-    launch_classify(cls_blocks, s, f32, fine, w, n, vec, t->hdr, t->agg, t->slist, ntiles);
-    if (tm) cudaEventRecord(t->ev[3], s);
-    k_tilescan<<<nchunks, kThreads, 0, s>>>(t->hdr, t->agg, t->cagg, t->cincl, t->incl, t->flags, ntiles, epoch,
-                                            wait_limit, skip_tile);
-    if (tm) cudaEventRecord(t->ev[4], s);
-    launch_split(s, fine, t->incl, ntiles, n, t->hdr, t->split);
-    if (o.acc == WRS_ACC_U64) k_require_u64<<<1, 32, 0, s>>>(t->hdr);
-    if (tm) cudaEventRecord(t->ev[5], s);
-    // a subproblem of the caller's split count (a run of tiles) is packed by one or more warps
-    const uint32_t group = sweep_group(ntiles, fine ? o.group * (kTile / kFineTile) : o.group);
-    launch_sweep(s, f32, fine, w, n, vec, t->hdr, t->split, t->slist, ntiles, t->buckets, group, o.acc == WRS_ACC_U128);
+    if (n <= (uint64_t)kTile) { // one launch; the stage times are 0 but the last
+        if (tm)
+            for (int i = 1; i < kStages; ++i) cudaEventRecord(t->ev[i], s);
+        launch_small(s, f32, w, n, vec, t->hdr, t->buckets, o.acc);
+    } else {
+        if (f32) k_stats<1><<<nparts, kThreads, 0, s>>>(w, n, vec, t->part);
+        else k_stats<0><<<nparts, kThreads, 0, s>>>(w, n, vec, t->part);
+        if (tm) cudaEventRecord(t->ev[1], s);
+        k_stats_combine<<<1, kThreads, 0, s>>>(t->part, nparts, n, f32, t->hdr);
+        if (tm) cudaEventRecord(t->ev[2], s);
+        launch_classify(cls_blocks, s, f32, fine, w, n, vec, t->hdr, t->agg, t->slist, ntiles);
+        if (tm) cudaEventRecord(t->ev[3], s);
+        k_tilescan<<<nchunks, kThreads, 0, s>>>(t->hdr, t->agg, t->cagg, t->cincl, t->incl, t->flags, ntiles, epoch,
+                                                wait_limit, skip_tile);
+        if (tm) cudaEventRecord(t->ev[4], s);
+        launch_split(s, fine, t->incl, ntiles, n, t->hdr, t->split);
+        if (o.acc == WRS_ACC_U64) k_require_u64<<<1, 32, 0, s>>>(t->hdr);
+        if (tm) cudaEventRecord(t->ev[5], s);
+        // a subproblem of the caller's split count (a run of tiles) is packed by one or more warps
+        const uint32_t group = sweep_group(ntiles, fine ? o.group * (kTile / kFineTile) : o.group);
+        launch_sweep(s, f32, fine, w, n, vec, t->hdr, t->split, t->slist, ntiles, t->buckets, group, o.acc == WRS_ACC_U128);
+    }
     if (tm) cudaEventRecord(t->ev[6], s);
     t->timed_build = tm;
     wrs_status st = launch_err();
@@ -829,6 +840,11 @@ extern "C" wrs_status wrs_build_noalloc(const void *d_weights, uint64_t n, wrs_d
     if (nparts > blocks_cap) nparts = blocks_cap;
     const uint32_t cls_want = (ntiles + kWarps - 1) / kWarps; // one warp per tile
     uint32_t cls_blocks = blocks_cap < cls_want ? blocks_cap : cls_want;
+    if (n <= (uint64_t)kTile) {
+        if (check_clear(buckets, n, s) != WRS_OK) return WRS_EDEVICE;
+        launch_small(s, f32, w, n, vec, hdr, buckets, WRS_ACC_AUTO);
+        return launch_err();
+    }
     // the look-back flags start from zero on the stream, in stream order with
     // the scan that reads them
     if (cudaMemsetAsync(flags, 0, (size_t)nchunks * sizeof(uint32_t), s) != cudaSuccess) return WRS_EDEVICE;

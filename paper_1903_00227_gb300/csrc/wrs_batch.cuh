@@ -71,28 +71,21 @@ __global__ void __launch_bounds__(kThreads) kb_stats_combine(const BatchTable *_
     stats_combine_body(part + T.part0, T.nparts, T.n, f32, hdr + blockIdx.x);
 }
 
-// A table of at most one tile, whole, in one block: validity, exact total
-// and lowest set bit (as k_stats + k_stats_combine), the header, then Alg. 2
-// on its n items with capacity Q and item weights n * q (group_build: the
-// table is a single group), and the light count.  The buckets and header
-// equal those of the tile pipeline.
+// A table of at most kTile weights, whole, in one block: validity, exact
+// total and lowest set bit (as k_stats + k_stats_combine), the header, then
+// Alg. 2 on its n items with capacity Q and item weights n * q (group_build:
+// the table is a single group), and the light count.  The buckets and header
+// equal those of the tile pipeline.  acc: a wrs_acc.
 template <int F32>
-__global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restrict__ w, int vec,
-                                                        const BatchTable *__restrict__ bt,
-                                                        const BlockMap *__restrict__ map, DevHeader *hdr_all,
-                                                        uint4 *__restrict__ buckets)
+__device__ __forceinline__ void small_build(const uint32_t *__restrict__ w, uint64_t N, int vec, DevHeader *hdr,
+                                            uint4 *__restrict__ buckets, int acc)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GroupSmem &S = *reinterpret_cast<GroupSmem *>(smem_raw);
     __shared__ uint32_t s_status;
-    const BlockMap m = map[blockIdx.x];
-    const BatchTable &T = bt[m.table];
-    DevHeader *hdr = hdr_all + m.table;
-    const uint64_t N = T.n;
-    const uint32_t *wt = w + T.off;
     const uint64_t first = (uint64_t)threadIdx.x * kItems;
     uint32_t x[kItems];
-    load_items(wt, N, vec, first, x);
+    load_items(w, N, vec, first, x);
     Acc a;
     a.base = F32 ? INT_MAX : 0;
     a.acc = 0;
@@ -108,7 +101,10 @@ __global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restri
     }
     acc_fold(a, a64);
     a = acc_block_reduce(a);
-    if (threadIdx.x == 0) s_status = write_header(a, N, F32, hdr);
+    if (threadIdx.x == 0) {
+        s_status = write_header(a, N, F32, hdr);
+        if (acc == WRS_ACC_U64 && s_status == 0 && hdr->q_hi != 0) s_status = hdr->status = kEOverflow;
+    }
     __syncthreads();
     if (s_status) return;
     const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
@@ -124,10 +120,32 @@ __global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restri
     uint32_t nl;
     block_exclusive_scan_u32(cl, nl, S.cnt);
     if (threadIdx.x == 0) hdr->n_light = nl;
-    const bool bad = bitlen128(Q) <= 52
-                         ? group_build<uint64_t>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets + T.off, hdr)
-                         : group_build<u128>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets + T.off, hdr);
+    const bool bad = bitlen128(Q) <= 52 && acc != WRS_ACC_U128
+                         ? group_build<uint64_t>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets, hdr)
+                         : group_build<u128>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets, hdr);
     if (bad) set_status(hdr, kEInternal);
+}
+
+template <int F32>
+__global__ void __launch_bounds__(kThreads, 3) kb_small(const uint32_t *__restrict__ w, int vec,
+                                                        const BatchTable *__restrict__ bt,
+                                                        const BlockMap *__restrict__ map, DevHeader *hdr,
+                                                        uint4 *__restrict__ buckets)
+{
+    const BlockMap m = map[blockIdx.x];
+    const BatchTable &T = bt[m.table];
+    small_build<F32>(w + T.off, T.n, vec, hdr + m.table, buckets + T.off, WRS_ACC_AUTO);
+}
+
+// A single table of at most kTile weights.  Bound by launches: the six
+// kernels of the tile pipeline take 41 us for 1500 weights, most of it their
+// start, end and one block's latency; this one replaces them all (1500 weights
+// built and 200 samples drawn: 46.8 -> 22.5 us a pass).
+template <int F32>
+__global__ void __launch_bounds__(kThreads, 3) k_small(const uint32_t *__restrict__ w, uint64_t n, int vec,
+                                                       DevHeader *hdr, uint4 *__restrict__ buckets, int acc)
+{
+    small_build<F32>(w, n, vec, hdr, buckets, acc);
 }
 
 template <int F32, int TILE>
@@ -315,6 +333,21 @@ wrs_status apply_groups(wrs_batch *b)
     wrs_status st = upload_map(b, kMapSweep, m);
     if (st == WRS_OK) st = upload_tables(b);
     return st;
+}
+
+wrs_status small_attributes()
+{
+    const int bytes = (int)sizeof(GroupSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_small<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e == cudaSuccess ? WRS_OK : WRS_EDEVICE;
+}
+
+void launch_small(cudaStream_t s, bool f32, const uint32_t *w, uint64_t n, int vec, DevHeader *hdr, uint4 *buckets,
+                  int acc)
+{
+    auto *k = f32 ? k_small<1> : k_small<0>;
+    k<<<1, kThreads, sizeof(GroupSmem), s>>>(w, n, vec, hdr, buckets, acc);
 }
 
 void batch_launch_sweep(wrs_batch *b, const uint32_t *w, int vec, bool f32, cudaStream_t s)

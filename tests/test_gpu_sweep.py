@@ -1,7 +1,7 @@
-"""The sweep at the edges of its dispatch: tile sizes (fine tiles up to 2^22
-weights), 32-, 96- and 128-bit key modes, dense and sparse heavies, long light
-runs, ragged ends, unaligned weights.  Tables are integers: equal to the
-oracle's, bucket for bucket."""
+"""The build at the edges of its dispatch: one launch up to 2048 weights, tile
+sizes (fine tiles up to 2^22 weights), the sweep's key modes, dense and sparse
+heavies, long light runs, ragged ends, unaligned weights.  Tables are integers:
+equal to the oracle's, bucket for bucket."""
 import numpy as np
 import pytest
 import torch
@@ -21,7 +21,7 @@ def _runs(n, rng):
     w = np.ones(n, np.float32)
     w[n // 5: n // 3] = 0
     w[n // 3: n // 2] = rng.random(n // 2 - n // 3).astype(np.float32) * 4
-    w[n // 2:: 700] = 900.0
+    w[n // 2::700] = 900.0
     return w
 
 
@@ -37,7 +37,7 @@ CASES = {
 
 
 @pytest.mark.parametrize("kind", CASES)
-@pytest.mark.parametrize("n", [2047, 257, FINE_MAX - 1, FINE_MAX, FINE_MAX + 1])
+@pytest.mark.parametrize("n", [1, 257, 2047, 2048, 2049, FINE_MAX - 1, FINE_MAX, FINE_MAX + 1])
 def test_sweep_matches_oracle(kind, n):
     w = CASES[kind](n)
     _, tab = O.build_table(w)
