@@ -110,19 +110,20 @@ __device__ __forceinline__ void small_build(const uint32_t *__restrict__ w, uint
     const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
     const int beta = hdr->beta;
     const uint32_t shift = hdr->shift;
-    u128 q[kItems];
-    uint32_t cl = 0;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        q[k] = first + k < N ? q_of(x[k], F32, beta) : (u128)0;
-        if (first + k < N && q[k] * (u128)N <= Q) ++cl;
-    }
+    bool bad;
     uint32_t nl;
-    block_exclusive_scan_u32(cl, nl, S.cnt);
+    if (bitlen128(Q) <= 52 && acc != WRS_ACC_U128) {
+        uint64_t q[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) q[k] = F32 ? q64_small(x[k], beta) : (uint64_t)x[k]; // 0 past the end
+        bad = group_build<uint64_t>(S, q, lo64(Q), (uint32_t)N, N, first, 0, shift, buckets, hdr, nl);
+    } else {
+        u128 q[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) q[k] = first + k < N ? q_of(x[k], F32, beta) : (u128)0;
+        bad = group_build<u128>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets, hdr, nl);
+    }
     if (threadIdx.x == 0) hdr->n_light = nl;
-    const bool bad = bitlen128(Q) <= 52 && acc != WRS_ACC_U128
-                         ? group_build<uint64_t>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets, hdr)
-                         : group_build<u128>(S, q, Q, (uint32_t)N, N, first, 0, shift, buckets, hdr);
     if (bad) set_status(hdr, kEInternal);
 }
 

@@ -47,13 +47,14 @@ __device__ __forceinline__ uint32_t swz(uint32_t j) { return j ^ ((j >> 3) & 7u)
 // keys and keeps the gap between the last probe before the answer and the
 // first one after it, so a range of 2048 takes two rounds and a final probe
 // of at most 32 keys.  Every lane returns the answer.
-__device__ __forceinline__ uint32_t warp_search(const u128 *key, uint32_t lo, uint32_t hi, u128 v, bool upper)
+template <typename K>
+__device__ __forceinline__ uint32_t warp_search(const K *key, uint32_t lo, uint32_t hi, K v, bool upper)
 {
     const uint32_t lane = threadIdx.x & 31;
     while (hi - lo > 32) {
         const uint32_t step = (hi - lo + 31) / 32;
         const uint32_t p = lo + step * lane;
-        const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
+        const bool before = p < hi && (upper ? key[swzk<K>(p)] <= v : key[swzk<K>(p)] < v);
         const uint32_t cnt = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before)); // probes before the answer
         if (cnt == 0) return lo;
         const uint32_t nhi = lo + step * cnt; // first probe not before the answer (or past hi)
@@ -61,7 +62,7 @@ __device__ __forceinline__ uint32_t warp_search(const u128 *key, uint32_t lo, ui
         hi = nhi < hi ? nhi : hi;
     }
     const uint32_t p = lo + lane;
-    const bool before = p < hi && (upper ? key[swz(p)] <= v : key[swz(p)] < v);
+    const bool before = p < hi && (upper ? key[swzk<K>(p)] <= v : key[swzk<K>(p)] < v);
     return lo + (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before));
 }
 
@@ -96,91 +97,50 @@ __device__ __forceinline__ u128 ld_key(const uint4 *p)
 }
 
 // ------------------------------------------------------------ phase 1
-template <int F32>
-__global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__restrict__ w, uint64_t n, int vec,
-                                                          DevHeader *hdr, uint4 *__restrict__ table,
-                                                          TileSum *__restrict__ tsum, uint4 *__restrict__ skeys,
-                                                          uint32_t *__restrict__ sidx)
+// Tile `tile` with keys of width K, words x (8 consecutive ones a thread).
+template <int F32, typename K>
+__device__ __forceinline__ bool pp_tile(GroupSmem &S, const uint32_t (&x)[kItems], uint64_t n, DevHeader *hdr,
+                                        uint32_t tile, uint4 *__restrict__ table, TileSum *__restrict__ tsum,
+                                        uint4 *__restrict__ skeys, uint32_t *__restrict__ sidx)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    GroupSmem &S = *reinterpret_cast<GroupSmem *>(smem_raw);
+    K *okey = reinterpret_cast<K *>(S.okey);
+    K *hkey = reinterpret_cast<K *>(S.hkey);
     __shared__ uint32_t s_ab[2];
-    __shared__ u128 s_res;
-    if (block_stopped(hdr)) return;
+    __shared__ K s_res;
     const uint32_t n32 = (uint32_t)n;
-    const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
+    const K Q = (K)mk128(hdr->q_lo, hdr->q_hi);
     const uint32_t light_max = hdr->light_max, shift = hdr->shift;
     const int beta = hdr->beta;
-    const uint32_t tile = blockIdx.x;
     const uint64_t tile0 = (uint64_t)tile * kTile;
     const uint64_t first = tile0 + (uint64_t)threadIdx.x * kItems;
-    uint32_t x[kItems];
-    load_items(w, n, vec, first, x);
+    K v[kItems];
     uint32_t lmask = 0, hmask = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
+        // 64-bit keys: n q < 2^51, so q < 2^51
+        v[k] = sizeof(K) == 8 ? (K)((F32 ? q64_small(x[k], beta) : (uint64_t)x[k]) * n32)
+                              : (K)nq_of(x[k], F32, beta, n32);
         if (first + k < n) {
             if (x[k] <= light_max) lmask |= 1u << k; else hmask |= 1u << k;
         }
     }
-    uint32_t tot;
-    const uint32_t ex = block_exclusive_scan_u32((uint32_t)__popc(lmask) | ((uint32_t)__popc(hmask) << 16), tot,
-                                                 S.cnt);
-    const uint32_t nl = tot & 0xFFFFu, nh = tot >> 16;
-    const uint32_t l0 = ex & 0xFFFFu, h0 = ex >> 16;
-    u128 sd = 0, se = 0;
-    {
-        uint32_t ls = l0, hs = h0;
-#pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            if (!(((lmask | hmask) >> k) & 1u)) continue;
-            const u128 nq = nq_of(x[k], F32, beta, n32);
-            const uint16_t off = (uint16_t)(threadIdx.x * kItems + k);
-            if ((lmask >> k) & 1u) {
-                const u128 d = Q - nq;
-                S.okey[swz(ls)] = d;
-                S.ooff[ls] = off;
-                sd += d;
-                ++ls;
-            } else {
-                const u128 e = nq - Q;
-                S.hkey[swz(hs)] = e;
-                S.hoff[hs] = off;
-                se += e;
-                ++hs;
-            }
-        }
-    }
-    U2 sums;
-    const U2 exs = block_exclusive_scan2(U2{sd, se}, sums, S.scan);
-    {
-        u128 kl = exs.a, ke = exs.b;
-        for (uint32_t j = 0; j < (uint32_t)__popc(lmask); ++j) {
-            const u128 d = S.okey[swz(l0 + j)];
-            S.okey[swz(l0 + j)] = kl;
-            kl += d;
-        }
-        for (uint32_t j = 0; j < (uint32_t)__popc(hmask); ++j) {
-            ke += S.hkey[swz(h0 + j)];
-            S.hkey[swz(h0 + j)] = ke;
-        }
-    }
-    const u128 D_tot = sums.a;
-    __syncthreads();
+    const OwnKeys<K> O = own_keys<K>(S, v, Q, lmask, hmask);
+    const uint32_t nl = O.nl, nh = O.nh, l0 = O.l0, h0 = O.h0;
+    const K D_tot = O.sums.a;
     // where the greedy pass stops: A lights and B heavies are packed
     if (threadIdx.x < 32) {
         uint32_t A = 0, B = 0;
         if (nh > 0) {
-            const u128 E_last = S.hkey[swz(nh - 1)];
-            if (E_last > D_tot) { A = nl; B = warp_search(S.hkey, 0, nh, D_tot, true); }
-            else { A = warp_search(S.okey, 0, nl, E_last, false); B = nh - 1; }
+            const K E_last = hkey[swzk<K>(nh - 1)];
+            if (E_last > D_tot) { A = nl; B = warp_search<K>(hkey, 0, nh, D_tot, true); }
+            else { A = warp_search<K>(okey, 0, nl, E_last, false); B = nh - 1; }
         }
         if (threadIdx.x == 0) {
             s_ab[0] = A;
             s_ab[1] = B;
             if (B < nh) { // residual of the heavy item current at the stop
-                const u128 DA = A < nl ? S.okey[swz(A)] : D_tot;
-                s_res = S.hkey[swz(B)] - DA + Q;
+                const K DA = A < nl ? okey[swzk<K>(A)] : D_tot;
+                s_res = hkey[swzk<K>(B)] - DA + Q;
             }
         }
     }
@@ -194,62 +154,21 @@ __global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__rest
     // D - D_A, the leftover heavies' excesses E - E_B, and heavy B adds
     // Q - res to the lights after it or res - Q before the heavies.
     const bool hasB = B < nh;
-    const u128 res = hasB ? s_res : (u128)0;
+    const K res = hasB ? s_res : (K)0;
     const bool Bl = hasB && res <= Q, Bh = hasB && res > Q;
     const uint32_t offB = hasB ? S.hoff[B] : 0xFFFFFFFFu;
-    const u128 DA = A < nl ? S.okey[swz(A)] : D_tot;
-    const u128 EB = hasB ? S.hkey[swz(B)] : (u128)0;
+    const K DA = A < nl ? okey[swzk<K>(A)] : D_tot;
+    const K EB = hasB ? hkey[swzk<K>(B)] : (K)0;
     const uint32_t ncl = (nl - A) + (Bl ? 1u : 0u);
     const uint32_t nch = hasB ? (nh - B - 1) + (Bh ? 1u : 0u) : 0u;
     if (threadIdx.x == 0) {
-        const u128 lsum = (D_tot - DA) + (Bl ? Q - res : (u128)0);
-        const u128 hsum = hasB ? (S.hkey[swz(nh - 1)] - EB) + (Bh ? res - Q : (u128)0) : (u128)0;
+        const u128 lsum = (u128)(D_tot - DA) + (Bl ? Q - res : (K)0);
+        const u128 hsum = hasB ? (u128)(hkey[swzk<K>(nh - 1)] - EB) + (Bh ? res - Q : (K)0) : (u128)0;
         TileSum a;
         a.l_lo = lo64(lsum); a.l_hi = hi64(lsum); a.h_lo = lo64(hsum); a.h_hi = hi64(hsum);
         a.cl = ncl; a.nheavy = nch; a.first_heavy = kNone; a.pad = 0;
         tilesum_st(tsum + tile, a);
         atomicAdd(reinterpret_cast<unsigned long long *>(&hdr->n_light), (unsigned long long)nl);
-    }
-    // the packed items, lights [0, A) and heavies [0, B), as one merge
-    const uint32_t M = A + B;
-    const uint32_t per = (M + kThreads - 1) / kThreads;
-    const uint32_t d0 = threadIdx.x * per;
-    if (d0 < M) {
-        uint32_t lo = d0 > A ? d0 - A : 0, hi = d0 < B ? d0 : B;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (S.hkey[swz(mid - 1)] <= S.okey[swz(d0 - mid)]) lo = mid; else hi = mid - 1;
-        }
-        uint32_t j = lo, i = d0 - lo;
-        const uint32_t steps = min(per, M - d0);
-        u128 ej = j < nh ? S.hkey[swz(j)] : (u128)0;
-        u128 di = i < nl ? S.okey[swz(i)] : D_tot;
-        for (uint32_t st = 0; st < steps; ++st) {
-            if ((j < B) && (i >= A || ej <= di)) { // heavy j: Q - (D_i - E_j), alias the next heavy (in the tile)
-                const u128 gap = di - ej;
-                if (gap > Q || j + 1 >= nh) bad = true;
-                const uint32_t me = (uint32_t)(tile0 + S.hoff[j]);
-                const uint32_t nx = (uint32_t)(tile0 + S.hoff[min(j + 1, nh - 1)]);
-                const uint32_t alias = gap == 0 ? me : nx;
-                const uint64_t thr = lo64((Q - gap) >> shift);
-                put_bucket(table, me, thr, alias, n, hdr);
-                ++j;
-                if (j < nh) ej = S.hkey[swz(j)];
-            } else { // light i: its own weight, alias the current heavy
-                const u128 dn = i + 1 < nl ? S.okey[swz(i + 1)] : D_tot;
-                const u128 nq = Q - (dn - di);
-                const uint32_t me = (uint32_t)(tile0 + S.ooff[i]);
-                uint32_t alias = me;
-                if (nq != Q) {
-                    if (j < nh) alias = (uint32_t)(tile0 + S.hoff[j]);
-                    else bad = true;
-                }
-                const uint64_t thr = lo64(nq >> shift);
-                put_bucket(table, me, thr, alias, n, hdr);
-                ++i;
-                di = dn;
-            }
-        }
     }
     // the leftovers' keys local to the tile, in its staging slots: lights
     // first (D = deficits of the tile's leftover lights before), then heavies
@@ -264,30 +183,94 @@ __global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__rest
                 if (lr >= A) {
                     const bool after = Bl && offB < off;
                     const uint64_t pos = tile0 + (lr - A) + (after ? 1u : 0u);
-                    st_key(skeys + pos, S.okey[swz(lr)] - DA + (after ? Q - res : (u128)0));
+                    st_key(skeys + pos, (u128)(K)(okey[swzk<K>(lr)] - DA + (after ? Q - res : (K)0)));
                     sidx[pos] = (uint32_t)(first + k);
                 }
                 ++lr;
             } else if ((hmask >> k) & 1u) {
                 if (hr == B) {
                     if (Bl) { // lr = the lights before it
-                        const u128 Dk = lr < nl ? S.okey[swz(lr)] : D_tot;
+                        const K Dk = lr < nl ? okey[swzk<K>(lr)] : D_tot;
                         const uint64_t pos = tile0 + (lr > A ? lr - A : 0u);
-                        st_key(skeys + pos, lr > A ? Dk - DA : (u128)0);
+                        st_key(skeys + pos, (u128)(K)(lr > A ? Dk - DA : (K)0));
                         sidx[pos] = (uint32_t)(first + k);
                     } else {
-                        st_key(skeys + hbase, res - Q);
+                        st_key(skeys + hbase, (u128)(K)(res - Q));
                         sidx[hbase] = (uint32_t)(first + k);
                     }
                 } else if (hr > B) {
                     const uint64_t pos = hbase + (hr - B - 1) + (Bh ? 1u : 0u);
-                    st_key(skeys + pos, S.hkey[swz(hr)] - EB + (Bh ? res - Q : (u128)0));
+                    st_key(skeys + pos, (u128)(K)(hkey[swzk<K>(hr)] - EB + (Bh ? res - Q : (K)0)));
                     sidx[pos] = (uint32_t)(first + k);
                 }
                 ++hr;
             }
         }
     }
+    // the packed items, lights [0, A) and heavies [0, B), as one merge
+    const uint32_t M = A + B;
+    const uint32_t per = (M + kThreads - 1) / kThreads;
+    const uint32_t d0 = threadIdx.x * per;
+    if (d0 < M) {
+        uint32_t lo = d0 > A ? d0 - A : 0, hi = d0 < B ? d0 : B;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (hkey[swzk<K>(mid - 1)] <= okey[swzk<K>(d0 - mid)]) lo = mid; else hi = mid - 1;
+        }
+        uint32_t j = lo, i = d0 - lo;
+        const uint32_t steps = min(per, M - d0);
+        K ej = j < nh ? hkey[swzk<K>(j)] : (K)0;
+        K di = i < nl ? okey[swzk<K>(i)] : D_tot;
+        for (uint32_t st = 0; st < steps; ++st) {
+            if ((j < B) && (i >= A || ej <= di)) { // heavy j: Q - (D_i - E_j), alias the next heavy (in the tile)
+                const K gap = di - ej;
+                if (gap > Q || j + 1 >= nh) bad = true;
+                const uint32_t me = S.hoff[j], nx = S.hoff[min(j + 1, nh - 1)];
+                put_bucket(table, tile0 + me, thr_of<K>(Q - gap, shift), (uint32_t)(tile0 + (gap == 0 ? me : nx)), n, hdr);
+                ++j;
+                if (j < nh) ej = hkey[swzk<K>(j)];
+            } else { // light i: its own weight, alias the current heavy
+                const K dn = i + 1 < nl ? okey[swzk<K>(i + 1)] : D_tot;
+                const K nq = Q - (dn - di);
+                const uint32_t me = S.ooff[i];
+                uint32_t alias = me;
+                if (nq != Q) {
+                    if (j < nh) alias = S.hoff[j];
+                    else bad = true;
+                }
+                put_bucket(table, tile0 + me, thr_of<K>(nq, shift), (uint32_t)(tile0 + alias), n, hdr);
+                ++i;
+                di = dn;
+            }
+        }
+    }
+    return bad;
+}
+
+// One tile per block.  64-bit keys when every n q of the tile and Q lie below
+// 2^51, so that its sums stay below 2^62 (n = 10^8 uniform weights do); other
+// tiles take 128 bits.  Bound by instruction issue: n = 10^8 uniform 1.40 ms
+// with 128-bit keys only (11.4 warp instructions per weight), 1.12 ms with
+// 64-bit keys (8.4), 1.00 ms with the keys written once (own_keys).
+template <int F32>
+__global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__restrict__ w, uint64_t n, int vec,
+                                                          DevHeader *hdr, uint4 *__restrict__ table,
+                                                          TileSum *__restrict__ tsum, uint4 *__restrict__ skeys,
+                                                          uint32_t *__restrict__ sidx)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    GroupSmem &S = *reinterpret_cast<GroupSmem *>(smem_raw);
+    if (block_stopped(hdr)) return;
+    uint32_t x[kItems];
+    load_items(w, n, vec, (uint64_t)blockIdx.x * kTile + (uint64_t)threadIdx.x * kItems, x);
+    uint32_t mx = 0;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) mx = max(mx, x[k]);
+    const u128 top = nq_of(mx, F32, hdr->beta, (uint32_t)n);
+    const bool narrow = bitlen128(mk128(hdr->q_lo, hdr->q_hi)) <= 51 && bitlen128(top) <= 51;
+    const bool bad = __syncthreads_and(narrow)
+                         ? pp_tile<F32, uint64_t>(S, x, n, hdr, blockIdx.x, table, tsum, skeys, sidx)
+                         : pp_tile<F32, u128>(S, x, n, hdr, blockIdx.x, table, tsum, skeys, sidx);
     if (bad) set_status(hdr, kEInternal);
 }
 

@@ -49,3 +49,31 @@ def test_sweep_matches_oracle(kind, n):
             assert t.status() == wrs.OK
             thr, alias, _ = t.download()
             assert np.array_equal(thr, tab.thr) and np.array_equal(alias, tab.alias)
+
+
+@pytest.mark.parametrize("kind", ["narrow", "wide", "mixed", "u32"])
+@pytest.mark.parametrize("n", [1, 2049, 3 * 2048, 40_007])
+def test_psa_plus_and_groups_in_both_key_widths(kind, n):
+    """Tiles and groups whose sums fit 64 bits stage their buckets, others
+    store them at once; a table may hold both kinds."""
+    if kind == "u32":
+        w = WL.u32_uniform(n, 12)
+    else:
+        w = WL.f32_uniform(n, 11)
+        if kind == "wide":  # n q up to 2^80
+            w = (w * np.float32(2.0) ** np.random.default_rng(13).integers(-20, 20, n)).astype(np.float32)
+        elif kind == "mixed":
+            w[::5000] = 2.0 ** 40
+    qz = O.quantize(w)
+    tab, left = O.psa_plus(qz, 2048, return_left=True)
+    with wrs.AliasTable(n) as t:
+        t.build_psa_plus(G.to_device(w))
+        assert t.status() == wrs.OK
+        thr, alias, _ = t.download()
+        assert np.array_equal(thr, tab.thr) and np.array_equal(alias, tab.alias)
+    ref = O.build_2lvl(qz)
+    with wrs.AliasTable2(n) as t2:
+        t2.build(G.to_device(w))
+        assert t2.status() == wrs.OK
+        thr, alias, *_ = t2.download()
+        assert np.array_equal(thr, ref.thr) and np.array_equal(alias, ref.alias)
