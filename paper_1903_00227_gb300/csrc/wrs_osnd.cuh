@@ -146,8 +146,8 @@ __device__ __forceinline__ double os_lfact(uint64_t k, double hl2pi)
     return ((double)k + 0.5) * os_log(z) - z + hl2pi + corr;
 }
 
-// Binomial(n, num / den), 0 < num < den
-__device__ uint64_t os_binomial(uint64_t n, u128 num, u128 den, OsRng &rng)
+// Binomial(n, num / den), 0 < num < den; hl2pi = 0.5 * os_log(2 pi)
+__device__ uint64_t os_binomial(uint64_t n, u128 num, u128 den, OsRng &rng, double hl2pi)
 {
     bool flip = false;
     if (2 * num > den) { num = den - num; flip = true; }
@@ -174,9 +174,9 @@ __device__ uint64_t os_binomial(uint64_t n, u128 num, u128 den, OsRng &rng)
         const double b = 1.15 + 2.53 * spq, a = -0.0873 + 0.0248 * b + 0.01 * p, c = (double)n * p + 0.5;
         const double vr = 0.92 - 4.2 / b, alpha = (2.83 + 5.1 / b) * spq;
         const uint64_t m = (uint64_t)floor(((double)n + 1.0) * p);
-        // log(p/q), log(m!) + log((n-m)!) and 0.5 log(2 pi) are needed only when
-        // the quick acceptance test fails: formed then, once (same values)
-        double lpq = 0.0, h = 0.0, hl2pi = 0.0;
+        // log(p/q) and log(m!) + log((n-m)!) are needed only when the quick
+        // acceptance test fails: formed then, once (same values)
+        double lpq = 0.0, h = 0.0;
         bool slow = false;
         for (;;) {
             const double u = os_unif(rng) - 0.5;
@@ -188,7 +188,6 @@ __device__ uint64_t os_binomial(uint64_t n, u128 num, u128 den, OsRng &rng)
             x = (uint64_t)kd;
             if (us >= 0.07 && v <= vr) break;
             if (!slow) {
-                hl2pi = 0.5 * os_log(6.283185307179586);
                 lpq = os_log(p / q);
                 h = os_lfact(m, hl2pi) + os_lfact(n - m, hl2pi);
                 slow = true;
@@ -200,17 +199,53 @@ __device__ uint64_t os_binomial(uint64_t n, u128 num, u128 den, OsRng &rng)
     return flip ? n - x : x;
 }
 
-struct OsNode {       // a node of a group's divide-and-conquer tree with samples
+// The first part of os_binomial for a node: kOsDone with the deviate in x;
+// kOsInvert for inversion (left to os_binomial from the start); kOsTry at the
+// first try of BTRS that the quick acceptance test does not settle, with that
+// try's Philox index in `tries`: os_binomial with rng.j set to it goes on from
+// there (a try takes one Philox call, so it draws the same numbers again).
+enum OsQuick { kOsDone, kOsInvert, kOsTry };
+__device__ __forceinline__ OsQuick os_binomial_quick(uint64_t n, u128 num, u128 den, OsRng &rng, uint64_t &x,
+                                                  uint32_t &tries)
+{
+    tries = 0;
+    bool flip = false;
+    if (2 * num > den) { num = den - num; flip = true; }
+    const double p = os_u128_to_double(num) / os_u128_to_double(den), q = 1.0 - p;
+    if ((double)n * p < 10.0) return kOsInvert;
+    const double spq = sqrt((double)n * p * q);
+    const double b = 1.15 + 2.53 * spq, a = -0.0873 + 0.0248 * b + 0.01 * p, c = (double)n * p + 0.5;
+    const double vr = 0.92 - 4.2 / b;
+    for (;;) {
+        tries = rng.j;
+        const double u = os_unif(rng) - 0.5;
+        const double v = os_unif(rng);
+        if (rng.j >= kOsMaxDraws) return kOsTry;
+        const double us = 0.5 - fabs(u);
+        const double kd = floor((2.0 * a / us + b) * u + c);
+        if (kd < 0.0 || kd > (double)n) continue;
+        if (!(us >= 0.07 && v <= vr)) return kOsTry;
+        x = flip ? n - (uint64_t)kd : (uint64_t)kd;
+        return kOsDone;
+    }
+}
+
+struct OsNode {       // an inner node of a group's divide-and-conquer tree with samples
     uint64_t c;
     uint16_t a, b, h, pad;
 };
+struct OsSlow {       // a node that the first pass did not settle
+    uint32_t node, tries;
+};
 
 struct OsSmem {
-    u128 pre[kTile + 1];      // prefix sums of the members' exact weights
-    OsNode node[2][kTile];    // nodes of the current and the next depth
+    u128 pre[kTile + 1];          // prefix sums of the members' exact weights
+    OsNode node[2][kTile / 2];    // inner nodes of the current and the next depth
+    OsSlow slow[kTile / 2];       // inversions from the front, tries from the back
     u128 red[kWarps];
     U2 scan[kWarps];
-    uint32_t nnode[2];
+    uint32_t nnode[2], ninvert, ntry;
+    double hl2pi;
     uint32_t pick[kOsBase];
     uint32_t cnt[kOsBase];
 };
@@ -226,6 +261,18 @@ __device__ __forceinline__ void os_emit(uint32_t *items, uint64_t *counts, unsig
 {
     const unsigned long long at = atomicAdd(nout, 1ull);
     if (at < cap) { items[at] = item; counts[at] = c; }
+}
+
+// os_emit for the lanes of a converged warp that have a pair: one atomic.
+__device__ __forceinline__ void os_emit_warp(uint32_t *items, uint64_t *counts, unsigned long long *nout,
+                                             uint64_t cap, bool on, uint32_t item, uint64_t c)
+{
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, on), lane = threadIdx.x & 31;
+    if (m == 0) return;
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(nout, (unsigned long long)__popc(m));
+    at = __shfl_sync(0xFFFFFFFFu, at, 0) + (unsigned long long)__popc(m & ((1u << lane) - 1u));
+    if (on && at < cap) { items[at] = item; counts[at] = c; }
 }
 
 // The top frontier (the single top group with all k samples) and zeroed counters.
@@ -255,7 +302,10 @@ __device__ __forceinline__ void os_push(uint32_t level, uint32_t member, uint64_
     else next[atomicAdd(nnext, 1ull)] = f;
 }
 
-// One frontier entry per block iteration.  SRC as k2_group.
+// One frontier entry per block iteration.  SRC as k2_group.  Bound by binary64
+// throughput (76 % of its pipe): n = 10^6 Zipf 1.0, k = 10^8 2.61 ms when each
+// thread finished its node's deviate on its own, 2.14 ms in two passes, 1.6 ms
+// with the second one's kinds apart.
 template <int SRC>
 __global__ void __launch_bounds__(kThreads) k_os_level(const void *__restrict__ src, int vec, uint64_t N,
                                                        uint32_t level, const uint4 *__restrict__ buckets,
@@ -274,6 +324,7 @@ __global__ void __launch_bounds__(kThreads) k_os_level(const void *__restrict__ 
     if (block_stopped(hdr)) return;
     const int beta = hdr->beta;
     const uint64_t nf = *nfront;
+    if (threadIdx.x == 0) S.hl2pi = 0.5 * os_log(6.283185307179586); // seen after the first barrier below
     for (uint64_t e = blockIdx.x; e < nf; e += gridDim.x) {
         const OsFront F = front[e];
         const uint32_t g = F.g;
@@ -346,43 +397,86 @@ __global__ void __launch_bounds__(kThreads) k_os_level(const void *__restrict__ 
             OsNode r;
             r.c = c; r.a = 0; r.b = (uint16_t)ng; r.h = 1; r.pad = 0;
             S.node[0][0] = r;
-            S.nnode[0] = 1;
+            S.nnode[0] = ng > 1;
             S.nnode[1] = 0;
+            S.ninvert = S.ntry = 0;
+            if (ng == 1) { // the group is a leaf
+                if (level == 0) os_emit(items, counts, nout, cap, (uint32_t)base, c);
+                else os_push(level, (uint32_t)base, c, next, nnext, next_small, nnext_small, N_next);
+            }
         }
         __syncthreads();
         int cur = 0;
-        while (S.nnode[cur] > 0) {
-            const uint32_t nn = S.nnode[cur];
-            for (uint32_t i = threadIdx.x; i < nn; i += kThreads) {
-                const OsNode d = S.node[cur][i];
-                if (d.b - d.a == 1) { // a leaf: an item, or a group one level down
-                    if (level == 0) os_emit(items, counts, nout, cap, (uint32_t)(base + d.a), d.c);
-                    else os_push(level, (uint32_t)(base + d.a), d.c, next, nnext, next_small, nnext_small, N_next);
-                    continue;
-                }
-                const uint32_t mid = d.a + (d.b - d.a) / 2;
-                const u128 wl = S.pre[mid] - S.pre[d.a], wn = S.pre[d.b] - S.pre[d.a];
-                uint64_t cl;
-                if (wl == 0) cl = 0;
-                else if (wl == wn) cl = d.c;
-                else {
-                    OsRng r;
-                    os_rng_init(r, seed, stream, g, d.h, level);
-                    cl = os_binomial(d.c, wl, wn, r);
-                }
-                if (cl) {
-                    OsNode l;
-                    l.c = cl; l.a = d.a; l.b = (uint16_t)mid; l.h = (uint16_t)(2 * d.h); l.pad = 0;
-                    S.node[cur ^ 1][atomicAdd(&S.nnode[cur ^ 1], 1u)] = l;
-                }
-                if (d.c - cl) {
-                    OsNode rr;
-                    rr.c = d.c - cl; rr.a = (uint16_t)mid; rr.b = d.b; rr.h = (uint16_t)(2 * d.h + 1); rr.pad = 0;
-                    S.node[cur ^ 1][atomicAdd(&S.nnode[cur ^ 1], 1u)] = rr;
+        // A node's samples to its children: cl of them to the left one.  Leaves
+        // (an item, or a group one level down) leave at once, so a depth holds
+        // inner nodes only.  Every thread of a warp calls; `on`: it has a node.
+        auto split = [&](const OsNode &d, uint64_t cl, bool on) {
+            const uint32_t mid = d.a + (d.b - d.a) / 2;
+#pragma unroll
+            for (int right = 0; right < 2; ++right) {
+                const uint32_t ca = right ? mid : d.a, cb = right ? d.b : mid;
+                const uint64_t cc = right ? d.c - cl : cl;
+                const bool has = on && cc != 0, leaf = has && cb - ca == 1;
+                if (level == 0) os_emit_warp(items, counts, nout, cap, leaf, (uint32_t)(base + ca), cc);
+                else if (leaf) os_push(level, (uint32_t)(base + ca), cc, next, nnext, next_small, nnext_small, N_next);
+                if (has && !leaf) {
+                    OsNode o;
+                    o.c = cc; o.a = (uint16_t)ca; o.b = (uint16_t)cb; o.h = (uint16_t)(2 * d.h + right); o.pad = 0;
+                    S.node[cur ^ 1][atomicAdd(&S.nnode[cur ^ 1], 1u)] = o;
                 }
             }
+        };
+        // Per depth in two passes: the deviates that BTRS's quick test settles,
+        // then the others, compacted by kind: inversion's exponential and the
+        // full test's logarithms cost two and six times as much binary64 work
+        // (what bounds this kernel), and a warp pays for every kind it holds.
+        while (S.nnode[cur] > 0) {
+            const uint32_t nn = S.nnode[cur];
+            for (uint32_t i0 = 0; i0 < nn; i0 += kThreads) {
+                const uint32_t i = i0 + threadIdx.x;
+                OsNode d{0, 0, 2, 0, 0};
+                bool on = i < nn;
+                uint64_t cl = 0;
+                if (on) {
+                    d = S.node[cur][i];
+                    const uint32_t mid = d.a + (d.b - d.a) / 2;
+                    const u128 wl = S.pre[mid] - S.pre[d.a], wn = S.pre[d.b] - S.pre[d.a];
+                    if (wl == 0) cl = 0;
+                    else if (wl == wn) cl = d.c;
+                    else {
+                        OsRng r;
+                        os_rng_init(r, seed, stream, g, d.h, level);
+                        uint32_t tries;
+                        const OsQuick st = os_binomial_quick(d.c, wl, wn, r, cl, tries);
+                        on = st == kOsDone;
+                        if (st == kOsInvert) S.slow[atomicAdd(&S.ninvert, 1u)] = OsSlow{i, 0};
+                        if (st == kOsTry) S.slow[kTile / 2 - 1 - atomicAdd(&S.ntry, 1u)] = OsSlow{i, tries};
+                    }
+                }
+                __syncwarp();
+                split(d, cl, on);
+            }
             __syncthreads();
-            if (threadIdx.x == 0) S.nnode[cur] = 0;
+            const uint32_t ni = S.ninvert, ni32 = (ni + 31) & ~31u, ns = ni32 + S.ntry; // a warp has one kind
+            for (uint32_t i0 = 0; i0 < ns; i0 += kThreads) {
+                const uint32_t i = i0 + threadIdx.x;
+                OsNode d{0, 0, 2, 0, 0};
+                const bool on = i < ni || (i >= ni32 && i < ns);
+                uint64_t cl = 0;
+                if (on) {
+                    const OsSlow sl = S.slow[i < ni ? i : kTile / 2 - 1 - (i - ni32)];
+                    d = S.node[cur][sl.node];
+                    const uint32_t mid = d.a + (d.b - d.a) / 2;
+                    OsRng r;
+                    os_rng_init(r, seed, stream, g, d.h, level);
+                    r.j = sl.tries;
+                    cl = os_binomial(d.c, S.pre[mid] - S.pre[d.a], S.pre[d.b] - S.pre[d.a], r, S.hl2pi);
+                }
+                __syncwarp();
+                split(d, cl, on);
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) { S.nnode[cur] = 0; S.ninvert = S.ntry = 0; }
             cur ^= 1;
             __syncthreads();
         }
@@ -488,7 +582,7 @@ wrs_status wrs_table2_sample_os(wrs_table2 *t, const void *d_weights, wrs_dtype 
                                k);
     if (k == 0) return launch_err();
     const size_t smem = sizeof(OsSmem);
-    const uint32_t cap_blocks = (uint32_t)sm_count() * 2;
+    const uint32_t cap_blocks = (uint32_t)sm_count() * 3; // by shared memory
     for (int l = (int)v.L - 1; l >= 0; --l) {
         const uint64_t lgroups = (v.size[l] + kTile - 1) / kTile;
         const uint32_t blocks = (uint32_t)(lgroups < cap_blocks ? lgroups : cap_blocks);
