@@ -36,7 +36,7 @@ struct wrs_table {
     uint64_t n;            // weights of the last build (0: never built)
     uint32_t epoch;        // look-back flag generation
     int device;
-    uint8_t *ws;           // workspace block
+    uint8_t *ws;           // workspace, behind the buckets in one allocation
     DevHeader *hdr;
     Partial *part;
     TileSum *agg, *incl;        // per tile
@@ -360,11 +360,14 @@ wrs_status launch_sample(const wrs_table *t, uint64_t s0, uint64_t s1, uint64_t 
 {
     const int sms = sm_count();
     const uint64_t k = s1 - s0;
-    uint64_t want = (k + 256ull * kSampleUnroll - 1) / (256ull * kSampleUnroll);
+    const bool small = t->n <= kSampleSmallN;
+    const uint64_t per_block = 256ull * (small ? kSampleUnrollSmall : kSampleUnroll);
+    uint64_t want = (k + per_block - 1) / per_block;
     uint64_t cap = (uint64_t)sms * 16; // 16 blocks per SM: more random loads in flight
     const uint32_t blocks = (uint32_t)(want < cap ? (want < 1 ? 1 : want) : cap);
-    k_sample<<<blocks, 256, 0, s>>>(t->buckets, t->n, t->hdr, s0, s1, (uint32_t)seed, (uint32_t)(seed >> 32),
-                                    (uint32_t)stream_id, (uint32_t)(stream_id >> 32), d_out);
+    auto *ks = small ? k_sample_small : k_sample;
+    ks<<<blocks, 256, 0, s>>>(t->buckets, t->n, t->hdr, s0, s1, (uint32_t)seed, (uint32_t)(seed >> 32),
+                              (uint32_t)stream_id, (uint32_t)(stream_id >> 32), d_out);
     return launch_err();
 }
 
@@ -403,19 +406,14 @@ wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out)
     cudaError_t e = cudaStreamCreateWithFlags(&t->log->priv, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->log->build_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) { destroy_log(t->log); delete t; return cuda_err(e); }
-    // stream-ordered allocations on the private stream, so that freeing the
+    // a stream-ordered allocation on the private stream, so that freeing the
     // table is stream-ordered too (cudaFreeAsync)
     cudaStream_t ps = t->log->priv;
-    e = cudaMallocAsync(reinterpret_cast<void **>(&t->ws), L.total, ps);
+    // (one block for both: a second one of a megabyte costs another mapping)
+    const uint64_t bucket_bytes = align_up(capacity_n * sizeof(uint4), 256);
+    e = cudaMallocAsync(reinterpret_cast<void **>(&t->buckets), bucket_bytes + L.total, ps);
     if (e != cudaSuccess) { destroy_log(t->log); delete t; return cuda_err(e); }
-    e = cudaMallocAsync(reinterpret_cast<void **>(&t->buckets), capacity_n * sizeof(uint4), ps);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(t->ws, ps);
-        cudaStreamSynchronize(ps);
-        destroy_log(t->log);
-        delete t;
-        return cuda_err(e);
-    }
+    t->ws = reinterpret_cast<uint8_t *>(t->buckets) + bucket_bytes;
     t->hdr = reinterpret_cast<DevHeader *>(t->ws + L.hdr);
     t->part = reinterpret_cast<Partial *>(t->ws + L.part);
     t->agg = reinterpret_cast<TileSum *>(t->ws + L.agg);
@@ -428,7 +426,6 @@ wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out)
     e = cudaMemsetAsync(t->ws, 0, L.total, ps);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ps);
     if (e != cudaSuccess) {
-        cudaFreeAsync(t->ws, ps);
         cudaFreeAsync(t->buckets, ps);
         cudaStreamSynchronize(ps);
         destroy_log(t->log);
@@ -694,7 +691,6 @@ void wrs_table_free(wrs_table *t)
         for (int i = 0; i <= kStages; ++i) cudaEventDestroy(t->ev[i]);
     if (t->copy_ev) cudaEventRecord(t->copy_ev, t->copy_stream);
     if (t->copy_ev) cudaStreamWaitEvent(ps, t->copy_ev, 0);
-    cudaFreeAsync(t->ws, ps);
     cudaFreeAsync(t->buckets, ps);
     if (t->stage_w) cudaFreeAsync(t->stage_w, ps);
     if (t->stage_out) cudaFreeAsync(t->stage_out, ps);

@@ -217,10 +217,11 @@ __global__ void __launch_bounds__(256) kb_sample(const BatchTable *__restrict__ 
 // Many sample requests against many resident tables in one launch.  Task i
 // draws k_i samples into out[out_offset_i ...]; the tasks' outputs are
 // consecutive (out_offset ascending, each the previous one plus its k).
-// Block b covers outputs [b * kManyPerBlock, ...): thread 0 finds the task
-// holding the first one by binary search, then the block walks the tasks
-// that overlap its range.  Sample s of a task is sample s of wrs_sample on
-// its table with the task's seed and stream id.
+// Block b covers outputs [b * kManyPerBlock, ...): its first warp finds the task
+// holding the first one (32 probes a round, so 1000 tasks take two dependent
+// reads instead of ten), then the block walks the tasks that overlap its range.
+// Sample s of a task is sample s of wrs_sample on its table with the task's
+// seed and stream id.
 constexpr uint32_t kManyPerBlock = 256 * 16;
 
 struct SampleTask {       // mirrors wrs_sample_task
@@ -234,19 +235,22 @@ static_assert(offsetof(SampleTask, hdr) == offsetof(wrs_sample_task, header), "l
 static_assert(offsetof(SampleTask, k) == offsetof(wrs_sample_task, k), "layout");
 static_assert(offsetof(SampleTask, out_offset) == offsetof(wrs_sample_task, out_offset), "layout");
 
-__global__ void __launch_bounds__(256) k_sample_many(const SampleTask *__restrict__ tasks, uint32_t ntasks,
+__global__ void __launch_bounds__(256, 4) k_sample_many(const SampleTask *__restrict__ tasks, uint32_t ntasks,
                                                      uint64_t total_k, uint32_t *__restrict__ out)
 {
     __shared__ uint32_t s_first;
     const uint64_t begin = (uint64_t)blockIdx.x * kManyPerBlock;
     const uint64_t end = min(begin + kManyPerBlock, total_k);
-    if (threadIdx.x == 0) { // last task with out_offset <= begin
+    if (threadIdx.x < 32) { // last task with out_offset <= begin; the first one's is at most begin
         uint32_t lo = 0, hi = ntasks - 1;
         while (lo < hi) {
-            const uint32_t mid = lo + (hi - lo + 1) / 2;
-            if (tasks[mid].out_offset <= begin) lo = mid; else hi = mid - 1;
+            const uint32_t step = (hi - lo + 31) / 32, p = lo + step * (threadIdx.x + 1);
+            const uint32_t cnt =
+                (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, p <= hi && p > lo && tasks[p].out_offset <= begin));
+            hi = min(hi, lo + step * (cnt + 1) - 1);
+            lo += step * cnt;
         }
-        s_first = lo;
+        if (threadIdx.x == 0) s_first = lo;
     }
     __syncthreads();
     for (uint32_t i = s_first; i < ntasks; ++i) {
@@ -255,7 +259,7 @@ __global__ void __launch_bounds__(256) k_sample_many(const SampleTask *__restric
         const uint64_t lo = max(begin, T.out_offset), hi = min(end, T.out_offset + T.k);
         if (lo >= hi || T.hdr->status) continue;
         // local sample indices [lo - off, hi - off), written at out + off + s
-        sample_body(T.buckets, T.n, T.hdr->qp, hi - T.out_offset, (uint32_t)T.seed, (uint32_t)(T.seed >> 32),
+        sample_body_small(T.buckets, T.n, T.hdr->qp, hi - T.out_offset, (uint32_t)T.seed, (uint32_t)(T.seed >> 32),
                     (uint32_t)T.stream_id, (uint32_t)(T.stream_id >> 32), out + T.out_offset,
                     lo - T.out_offset + threadIdx.x, 256);
     }

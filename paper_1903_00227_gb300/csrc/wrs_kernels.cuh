@@ -1239,7 +1239,15 @@ __device__ __forceinline__ uint4 ld_bucket(const uint4 *p)
     return v;
 }
 
-constexpr int kSampleUnroll = 8;
+// Queries a thread has in flight.  A table beyond the L2 is bound by random
+// DRAM reads (48 * 10^9 a second): 8 in flight at 102 registers, two blocks per
+// SM (3 10^8 samples of 10^9 buckets 6.28 ms; the code below for small tables
+// with 8 in flight at one, two or three blocks 6.34, 6.42, 6.55).  A table in the L2
+// is bound by the L1's one line per cycle and the arithmetic: 4 in flight,
+// 32-bit indices and no bounds tests in full rounds, so that twice the warps
+// fit (10^8 samples of 300,000 buckets 0.48 -> 0.39 ms).
+constexpr int kSampleUnroll = 8, kSampleUnrollSmall = 4;
+constexpr uint64_t kSampleSmallN = 1ull << 22; // 64 MB of buckets
 
 // Samples first, first + stride, ... (below k) of one table.
 __device__ __forceinline__ void sample_body(const uint4 *__restrict__ tab, uint64_t n, uint64_t qp, uint64_t k,
@@ -1276,6 +1284,43 @@ __device__ __forceinline__ void sample_body(const uint4 *__restrict__ tab, uint6
     }
 }
 
+// The same from a table that fits the L2.
+__device__ __forceinline__ void sample_body_small(const uint4 *__restrict__ tab, uint64_t n, uint64_t qp, uint64_t k,
+                                            uint32_t key0, uint32_t key1, uint32_t sid0, uint32_t sid1,
+                                            uint32_t *__restrict__ out, uint64_t first, uint64_t stride,
+                                            const DevHeader *chk = nullptr)
+{
+    const uint32_t n32 = (uint32_t)n; // n < 2^32
+    for (uint64_t s = first; s < k; s += kSampleUnrollSmall * stride) {
+        const bool all = s + (kSampleUnrollSmall - 1) * stride < k;
+        uint32_t r[kSampleUnrollSmall];
+        uint64_t v[kSampleUnrollSmall];
+        uint4 b[kSampleUnrollSmall];
+#pragma unroll
+        for (int j = 0; j < kSampleUnrollSmall; ++j) {
+            const uint64_t sj = s + j * stride;
+            P4 c;
+            c.x0 = (uint32_t)sj; c.x1 = (uint32_t)(sj >> 32); c.x2 = sid0; c.x3 = sid1;
+            const P4 o = philox4x32_10(c, key0, key1);
+            v[j] = o.x2 | ((uint64_t)o.x3 << 32);
+            r[j] = (uint32_t)(((uint64_t)o.x1 * n32 + __umulhi(o.x0, n32)) >> 32); // floor(u n / 2^64)
+        }
+#pragma unroll
+        for (int j = 0; j < kSampleUnrollSmall; ++j)
+            if (all || s + j * stride < k) b[j] = ld_bucket(tab + r[j]);
+#pragma unroll
+        for (int j = 0; j < kSampleUnrollSmall; ++j) {
+            const uint64_t sj = s + j * stride;
+            if (all || sj < k) {
+                const uint64_t thr = b[j].x | ((uint64_t)b[j].y << 32);
+                if (WRS_CHECK && chk) check_ok(b[j].z < n, const_cast<DevHeader *>(chk));
+                const uint32_t pick = (__umul64hi(v[j], qp) < thr) ? r[j] : b[j].z;
+                __stcs(out + sj, pick);
+            }
+        }
+    }
+}
+
 // Samples [s0, k) of one table.
 __global__ void __launch_bounds__(256) k_sample(const uint4 *__restrict__ tab, uint64_t n,
                                                 const DevHeader *__restrict__ hdr, uint64_t s0, uint64_t k,
@@ -1285,6 +1330,16 @@ __global__ void __launch_bounds__(256) k_sample(const uint4 *__restrict__ tab, u
     if (hdr->status) return;
     sample_body(tab, n, hdr->qp, k, key0, key1, sid0, sid1, out,
                 s0 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x, hdr);
+}
+
+__global__ void __launch_bounds__(256, 4) k_sample_small(const uint4 *__restrict__ tab, uint64_t n,
+                                                         const DevHeader *__restrict__ hdr, uint64_t s0, uint64_t k,
+                                                         uint32_t key0, uint32_t key1, uint32_t sid0, uint32_t sid1,
+                                                         uint32_t *__restrict__ out)
+{
+    if (hdr->status) return;
+    sample_body_small(tab, n, hdr->qp, k, key0, key1, sid0, sid1, out,
+                      s0 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x, hdr);
 }
 
 } // namespace wrs
