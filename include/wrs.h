@@ -110,7 +110,7 @@ wrs_status wrs_table_build(wrs_table *t, const void *d_weights, uint64_t n,
  *   splits  number of subproblems of Alg. 3's pack, each a run of
  *           consecutive 2048-weight tiles; 0: the library's choice; at most
  *           the number of tiles, ceil(n / 2048).  A run is packed by one warp
- *           of the sweep, or by several where the runs are longer than eight
+ *           of the sweep, or by several where the runs are longer than four
  *           tiles or too few to fill the GPU
  *   tile    0 or 2048 (fixed)
  *   window  0 or 2048 (fixed)
@@ -338,7 +338,7 @@ wrs_status wrs_batch_download(const wrs_batch *b, void *h_buckets, uint64_t byte
 
 /* Autotuning of the sweep.  Tables fall in WRS_BATCH_CLASSES size classes by
  * tiles of 2048 weights (1, 2-4, 5-32, 33-256, more); within a class every
- * sweep warp takes `group` consecutive tiles of one table, at most 8 (the
+ * sweep warp takes `group` consecutive tiles of one table, at most 4 (the
  * number of split subproblems of a table is its tiles / group; a batch of at
  * most 2^22 weights in all is cut into tiles of 256).  wrs_batch_tune builds
  * the batch from d_weights, then for each class present times the sweep

@@ -257,7 +257,7 @@ wrs_status read_back(const wrs_table *t, void *h, const void *d, size_t bytes)
     return cuda_err(e);
 }
 
-// Build options after validation: own tiles per sweep block (one subproblem
+// Build options after validation: own tiles per sweep warp (one subproblem
 // of Alg. 3 each), the accumulator mode.
 struct BuildOpts {
     uint32_t group = kSweepTiles;

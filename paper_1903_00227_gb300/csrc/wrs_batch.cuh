@@ -26,7 +26,7 @@ struct BatchTable {       // per table (device copy in wrs_batch::d_tables)
     uint64_t n;
     uint32_t ntiles, tile0;   // tiles, first tile in the per-tile arrays
     uint32_t part0, nparts;   // k_stats partials
-    uint32_t chunk0, group;   // first look-back chunk; own tiles per sweep block
+    uint32_t chunk0, group;   // first look-back chunk; own tiles per sweep warp
     uint64_t k, k_off;        // samples of the current plan, first output
     uint32_t sblocks, pad;    // blocks of the sampler
 };
@@ -36,7 +36,7 @@ struct BlockMap {         // one per block of a batch launch
 };
 
 constexpr int kBatchClasses = WRS_BATCH_CLASSES; // sweep size classes by tiles: 1, 2-4, 5-32, 33-256, more
-constexpr uint32_t kBatchGroups[] = {1, 2, 4, 8}; // tuner's candidates for own tiles per sweep block
+constexpr uint32_t kBatchGroups[] = {1, 2, 4, 8}; // tuner's candidates for own tiles per sweep warp
 constexpr uint32_t kBatchPartWeights = 16384;    // weights per k_stats block (at least)
 
 inline int batch_class(uint64_t n)

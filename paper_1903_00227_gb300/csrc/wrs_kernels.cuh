@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kThreads) k_split(const TileSum *__restrict__ 
 // block per eight tiles with 128-bit keys of a whole tile in shared memory, a
 // merge walked by threads and five barriers a tile.  n = 10^8, uniform / Zipf
 // 0.8 / Zipf 1.5: 1.54 / 1.50 / 1.18 -> 1.18 / 1.22 / 0.42 ms; n = 10^9 uniform
-// 15.4 -> 11.2 ms, Zipf 1.5 12.2 -> 3.3 ms.  One warp per block: the scheduler
+// 15.4 -> 10.9 ms, Zipf 1.5 12.2 -> 3.6 ms.  One warp per block: the scheduler
 // replaces each warp as it ends, 19 -> 23 resident warps per SM (1.47 -> 1.40 ms
 // uniform).  The rings fit 24 warps per SM, the registers (80) too.
 __device__ __forceinline__ uint4 split_head(const Split *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
@@ -842,7 +842,13 @@ template <typename K> __device__ __forceinline__ K split_E(const Split *p)
 }
 
 constexpr uint32_t kDirect = 128;        // weights a warp packs at once under one far heavy
-constexpr int kSweepTiles = 8;           // own tiles per task at most (the 32-bit keys cover 2^14 Q)
+// Own tiles per task at most.  More tiles share a task's start (its split
+// record, its first heavies' tile), fewer leave a shorter last wave and lights
+// and heavies that lie closer together: 1 / 2 / 4 / 8 / 16 tiles take 6.45 /
+// 6.38 / 6.62 / 6.90 / 7.36 ms for n = 6*10^8 uniform, 3.83 / 3.61 / 3.57 /
+// 3.61 / 3.81 ms for n = 10^9 Zipf 1.5, and 6.98 / 6.63 / 6.54 / 6.57 / - ms
+// for n = 6*10^8 Zipf 0.8.  (The 32-bit keys would cover 2^14 Q, eight tiles.)
+constexpr int kSweepTiles = 4;
 
 template <int F32, int MODE, int TILE>
 __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *__restrict__ w, uint64_t n, int vec,
