@@ -305,9 +305,14 @@ __device__ __forceinline__ void os_push(uint32_t level, uint32_t member, uint64_
 // One frontier entry per block iteration.  SRC as k2_group.  Bound by binary64
 // throughput (76 % of its pipe): n = 10^6 Zipf 1.0, k = 10^8 2.61 ms when each
 // thread finished its node's deviate on its own, 2.14 ms in two passes, 1.6 ms
-// with the second one's kinds apart.
+// with the second one's kinds apart.  Where a group's samples fall on few of
+// its items, by the latency of a depth: three blocks per SM, as many as the
+// shared memory allows, need at most 80 registers.  A call at n = 10^8 Zipf 1.5,
+// k = 10^9: 15.5 ms when two of the grid's three blocks per SM fit (102
+// registers), 12.5 with a grid of two, 9.1 with three (12.3 before the two
+// passes); n = 10^6 Zipf 1.0, k = 10^8 1.92 / 1.93 / 2.00 (2.94).
 template <int SRC>
-__global__ void __launch_bounds__(kThreads) k_os_level(const void *__restrict__ src, int vec, uint64_t N,
+__global__ void __launch_bounds__(kThreads, 3) k_os_level(const void *__restrict__ src, int vec, uint64_t N,
                                                        uint32_t level, const uint4 *__restrict__ buckets,
                                                        const GroupRec *__restrict__ groups, DevHeader *hdr,
                                                        const OsFront *__restrict__ front,
