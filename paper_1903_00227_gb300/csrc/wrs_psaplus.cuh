@@ -97,10 +97,12 @@ __device__ __forceinline__ u128 ld_key(const uint4 *p)
 }
 
 // ------------------------------------------------------------ phase 1
-// Tile `tile` with keys of width K, words x (8 consecutive ones a thread).
+// Tile `tile` with keys of width K, words x (8 consecutive ones a thread).  The
+// header's fields come from the caller, which loads them beside x: read here,
+// behind its barrier, they cost each tile one more trip to the L2.
 template <int F32, typename K>
 __device__ __forceinline__ bool pp_tile(GroupSmem &S, const uint32_t (&x)[kItems], uint64_t n, DevHeader *hdr,
-                                        uint32_t tile, uint4 *__restrict__ table, TileSum *__restrict__ tsum,
+                                        K Q, uint32_t light_max, uint32_t shift, int beta, uint32_t tile, uint4 *__restrict__ table, TileSum *__restrict__ tsum,
                                         uint4 *__restrict__ skeys, uint32_t *__restrict__ sidx)
 {
     K *okey = reinterpret_cast<K *>(S.okey);
@@ -108,9 +110,6 @@ __device__ __forceinline__ bool pp_tile(GroupSmem &S, const uint32_t (&x)[kItems
     __shared__ uint32_t s_ab[2];
     __shared__ K s_res;
     const uint32_t n32 = (uint32_t)n;
-    const K Q = (K)mk128(hdr->q_lo, hdr->q_hi);
-    const uint32_t light_max = hdr->light_max, shift = hdr->shift;
-    const int beta = hdr->beta;
     const uint64_t tile0 = (uint64_t)tile * kTile;
     const uint64_t first = tile0 + (uint64_t)threadIdx.x * kItems;
     K v[kItems];
@@ -251,7 +250,9 @@ __device__ __forceinline__ bool pp_tile(GroupSmem &S, const uint32_t (&x)[kItems
 // 2^51, so that its sums stay below 2^62 (n = 10^8 uniform weights do); other
 // tiles take 128 bits.  Bound by instruction issue: n = 10^8 uniform 1.40 ms
 // with 128-bit keys only (11.4 warp instructions per weight), 1.12 ms with
-// 64-bit keys (8.4), 1.00 ms with the keys written once (own_keys).
+// 64-bit keys (8.4), 1.00 ms with the keys written once (own_keys); the whole
+// build 1.41 -> 1.35 ms with the header read beside the weights (Zipf 1.5, on
+// 128-bit keys: 3.10 -> 2.98 ms, as before the two widths).
 template <int F32>
 __global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__restrict__ w, uint64_t n, int vec,
                                                           DevHeader *hdr, uint4 *__restrict__ table,
@@ -261,16 +262,19 @@ __global__ void __launch_bounds__(kThreads, 3) k_pp_local(const uint32_t *__rest
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GroupSmem &S = *reinterpret_cast<GroupSmem *>(smem_raw);
     if (block_stopped(hdr)) return;
+    const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
+    const uint32_t light_max = hdr->light_max, shift = hdr->shift;
+    const int beta = hdr->beta;
     uint32_t x[kItems];
     load_items(w, n, vec, (uint64_t)blockIdx.x * kTile + (uint64_t)threadIdx.x * kItems, x);
     uint32_t mx = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) mx = max(mx, x[k]);
-    const u128 top = nq_of(mx, F32, hdr->beta, (uint32_t)n);
-    const bool narrow = bitlen128(mk128(hdr->q_lo, hdr->q_hi)) <= 51 && bitlen128(top) <= 51;
+    const u128 top = nq_of(mx, F32, beta, (uint32_t)n);
+    const bool narrow = bitlen128(Q) <= 51 && bitlen128(top) <= 51;
     const bool bad = __syncthreads_and(narrow)
-                         ? pp_tile<F32, uint64_t>(S, x, n, hdr, blockIdx.x, table, tsum, skeys, sidx)
-                         : pp_tile<F32, u128>(S, x, n, hdr, blockIdx.x, table, tsum, skeys, sidx);
+                         ? pp_tile<F32, uint64_t>(S, x, n, hdr, (uint64_t)Q, light_max, shift, beta, blockIdx.x, table, tsum, skeys, sidx)
+                         : pp_tile<F32, u128>(S, x, n, hdr, Q, light_max, shift, beta, blockIdx.x, table, tsum, skeys, sidx);
     if (bad) set_status(hdr, kEInternal);
 }
 
