@@ -105,14 +105,13 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
+_CSRC = "paper_1903_00227_gb300/csrc/"
+_PSA = (_CSRC + "wrs_kernels.cuh", _CSRC + "wrs_pack.cuh", _CSRC + "wrs_device.cuh")
 KERNEL_SOURCES = {  # the files each measured kernel is compiled from
-    "psa": ("paper_1903_00227_gb300/csrc/wrs_kernels.cuh", "paper_1903_00227_gb300/csrc/wrs_device.cuh"),
-    "two_level": ("paper_1903_00227_gb300/csrc/wrs_kernels.cuh", "paper_1903_00227_gb300/csrc/wrs_device.cuh",
-                  "paper_1903_00227_gb300/csrc/wrs_twolevel.cuh"),
-    "os_nd": ("paper_1903_00227_gb300/csrc/wrs_kernels.cuh", "paper_1903_00227_gb300/csrc/wrs_device.cuh",
-              "paper_1903_00227_gb300/csrc/wrs_twolevel.cuh", "paper_1903_00227_gb300/csrc/wrs_osnd.cuh"),
-    "psa_plus": ("paper_1903_00227_gb300/csrc/wrs_kernels.cuh", "paper_1903_00227_gb300/csrc/wrs_device.cuh",
-                 "paper_1903_00227_gb300/csrc/wrs_twolevel.cuh", "paper_1903_00227_gb300/csrc/wrs_psaplus.cuh"),
+    "psa": _PSA,
+    "two_level": _PSA + (_CSRC + "wrs_twolevel.cuh",),
+    "os_nd": _PSA + (_CSRC + "wrs_twolevel.cuh", _CSRC + "wrs_osnd.cuh"),
+    "psa_plus": _PSA + (_CSRC + "wrs_twolevel.cuh", _CSRC + "wrs_psaplus.cuh"),
 }
 
 

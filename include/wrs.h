@@ -213,7 +213,8 @@ wrs_status wrs_table_upload(wrs_table *t, const void *h_buckets, uint64_t n,
 
 /* Stage timing: when enabled, every later build records CUDA events on its
  * stream between its six kernels (weight total, total combine, tile
- * classification, look-back scan of the tile sums, split search, sweep).
+ * classification, look-back scan of the tile sums, split search, sweep); a
+ * build of at most 2048 weights is one kernel, counted as the sweep.
  * wrs_table_stage_ms waits for the last build and writes the first `count`
  * (<= 6) stage durations in milliseconds.
  * Enabling creates the events (no device memory); errors: WRS_EINVAL when

@@ -822,8 +822,8 @@ __global__ void __launch_bounds__(kThreads) k_split(const TileSum *__restrict__ 
 // (its key is that far ahead), the lights go straight from the loaded words to
 // their buckets: Zipf 1.5 has 2000 lights per heavy.
 //
-// Bound by instruction issue (n = 10^8 uniform: 10.2 warp instructions per
-// weight at 71 % issue; about 290 per batch of own weights, 320 per batch of
+// Bound by instruction issue (n = 10^8 uniform: 9.5 warp instructions per
+// weight at 70 % issue; about 290 per batch of own weights, 320 per batch of
 // heavies' tile, 115 per search and 64 per 32 buckets stored).  It replaces a
 // block per eight tiles with 128-bit keys of a whole tile in shared memory, a
 // merge walked by threads and five barriers a tile.  n = 10^8, uniform / Zipf

@@ -6,10 +6,10 @@
 // light i; E[j]: excesses of the heavies up to and including heavy j) Alg. 2
 // is a merge of the two key sequences, heavy j before light i iff
 // E[j] <= D[i].  A warp keeps the next lights and heavies with their keys in
-// two rings in shared memory and emits 32 buckets a step: lane l finds the
-// heavies before light l among the next 32 by a five-step shuffle search, one
-// OR-reduction gives the merged order, and lane p writes the bucket of the
-// p-th item.  So a step costs the same whatever the mix of lights and
+// two rings in shared memory and emits up to 63 buckets a step: lane l finds
+// the heavies before light l among the next 32 by a five-step shuffle search,
+// one OR-reduction gives the merged order, and lane p writes the buckets of the
+// p-th and the (32 + p)-th item.  So a step costs the same whatever the mix of lights and
 // heavies, no lane idles, a warp's stores go to near positions (16-byte
 // stores by lanes that each own a run of items cost 6.7 to 10 ms per 10^9
 // buckets on a GB300, consecutive ones 2.1 ms), and no warp waits for another.
