@@ -868,6 +868,9 @@ __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *_
     bool bad = false;
 
     // lights: ranks [li, lh) are in the ring, weights from `at` on are not read yet (x: the next batch)
+    // Words past `end` read as 0xFFFFFFFF.  No binary32 table has a light threshold
+    // that high, but u32 weights that are all 0xFFFFFFFF have: there the last
+    // batch's words are told apart by their index.
     uint64_t at = (uint64_t)c_first * kTile;
     const uint64_t end = min((uint64_t)c_last * kTile, n);
     uint32_t li = 0, lh = 0, x[kPer];
@@ -928,7 +931,7 @@ __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *_
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        if (z[k] <= light_max) {
+                        if (z[k] <= light_max && (F32 || at + 32 * k + lane < end)) {
                             const K96 nq = U.nq_light(z[k]);
                             const K96 df = ksub(Ql, nq);
                             sum = kadd96(sum, df);
@@ -957,7 +960,8 @@ __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *_
                 uint32_t m = 0;
 #pragma unroll
                 for (int k = 0; k < kPer; ++k)
-                    if (x[k] <= light_max) m |= 1u << k; // past the end: never light
+                    if (x[k] <= light_max) m |= 1u << k;
+                if (!F32 && at + kBatch > end) m &= lane_words<kPer>(at, end); // the fill may be light
                 Light<MODE> v[kPer];
                 K sum{0, 0};
 #pragma unroll

@@ -446,6 +446,13 @@ __device__ __forceinline__ void load_lane(const uint32_t *__restrict__ w, int ve
     }
 }
 
+// Bit k: weight at + N lane + k lies below `end`.
+template <int N> __device__ __forceinline__ uint32_t lane_words(uint64_t at, uint64_t end)
+{
+    const uint64_t i = at + N * (threadIdx.x & 31);
+    return i >= end ? 0u : (1u << min((uint64_t)N, end - i)) - 1u;
+}
+
 // Ranks of this lane's members (mask m, bit k: item k) among the warp's, in
 // item order; tot: the warp's members.
 template <int N> __device__ __forceinline__ uint32_t warp_rank(uint32_t m, uint32_t &tot)
