@@ -62,33 +62,8 @@ struct wrs_table {
 
 namespace {
 
-constexpr uint32_t kMaxParts = 2048;     // blocks of k_stats
 std::atomic<uint32_t> g_wait_limit{1u << 22};
 std::atomic<int64_t> g_skip_tile{-1};
-
-inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
-
-struct Layout {
-    uint64_t hdr, part, agg, incl, cagg, cincl, flags, split, slist, total;
-};
-
-Layout layout_for(uint32_t ntiles, uint64_t slist_bytes)
-{
-    const uint32_t nchunks = (ntiles + kScanChunk - 1) / kScanChunk;
-    Layout L;
-    uint64_t o = 0;
-    L.hdr = o; o = align_up(o + sizeof(DevHeader), 256);
-    L.part = o; o = align_up(o + kMaxParts * sizeof(Partial), 256);
-    L.agg = o; o = align_up(o + (uint64_t)ntiles * sizeof(TileSum), 256);
-    L.incl = o; o = align_up(o + (uint64_t)ntiles * sizeof(TileSum), 256);
-    L.cagg = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
-    L.cincl = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
-    L.flags = o; o = align_up(o + (uint64_t)nchunks * sizeof(uint32_t), 256);
-    L.split = o; o = align_up(o + ((uint64_t)ntiles + 1) * sizeof(Split), 256);
-    L.slist = o; o = align_up(o + slist_bytes, 256);
-    L.total = o;
-    return L;
-}
 
 inline wrs_status cuda_err(cudaError_t e)
 {
@@ -120,29 +95,6 @@ int sm_count()
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms > 0 ? sms : 1;
-}
-
-// Tiles of n weights: kFineTile weights each up to kFineMax (below, a sweep
-// warp per 2048 weights leaves most of the GPU idle: n = 10^6 has 489 of them
-// for 3648 resident warps), else kTile.
-inline bool fine_tiles(uint64_t n) { return n <= kFineMax; }
-inline uint32_t tile_count(uint64_t n)
-{
-    const uint64_t tile = fine_tiles(n) ? kFineTile : kTile;
-    return (uint32_t)((n + tile - 1) / tile);
-}
-// Most tiles, and list bytes, that a build of at most `cap` weights has.
-inline uint32_t tiles_cap(uint64_t cap)
-{
-    const uint32_t fine = tile_count(cap < kFineMax ? cap : kFineMax);
-    const uint32_t all = tile_count(cap);
-    return fine > all ? fine : all;
-}
-inline uint64_t slist_cap(uint64_t cap)
-{
-    const uint64_t fine = (uint64_t)tile_count(cap < kFineMax ? cap : kFineMax) * kSparseOf(kFineTile);
-    const uint64_t all = fine_tiles(cap) ? fine : (uint64_t)tile_count(cap) * kSparseOf(kTile);
-    return (fine > all ? fine : all) * sizeof(uint16_t);
 }
 
 // Own tiles per task of the sweep (a warp each), at most `most`: as many as
@@ -402,7 +354,7 @@ wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out)
     t->cap = capacity_n;
     t->host_status = -1;
     cudaGetDevice(&t->device);
-    const Layout L = layout_for(tiles_cap(capacity_n), slist_cap(capacity_n));
+    const Layout L = layout_for(capacity_n);
     cudaError_t e = cudaStreamCreateWithFlags(&t->log->priv, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->log->build_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) { destroy_log(t->log); delete t; return cuda_err(e); }
@@ -410,7 +362,7 @@ wrs_status wrs_table_create(uint64_t capacity_n, wrs_table **out)
     // table is stream-ordered too (cudaFreeAsync)
     cudaStream_t ps = t->log->priv;
     // (one block for both: a second one of a megabyte costs another mapping)
-    const uint64_t bucket_bytes = align_up(capacity_n * sizeof(uint4), 256);
+    const uint64_t bucket_bytes = bucket_area(capacity_n);
     e = cudaMallocAsync(reinterpret_cast<void **>(&t->buckets), bucket_bytes + L.total, ps);
     if (e != cudaSuccess) { destroy_log(t->log); delete t; return cuda_err(e); }
     t->ws = reinterpret_cast<uint8_t *>(t->buckets) + bucket_bytes;

@@ -72,6 +72,59 @@ struct Split {              // result of k_split per tile boundary (48 B; ntiles
     uint64_t e_lo, e_hi;    // E after the heavies before this tile
 };
 
+// ------------------------------------- device memory of a table (host side)
+constexpr uint32_t kMaxParts = 2048;        // blocks of k_stats
+inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
+
+// Tiles of n weights: kFineTile weights each up to kFineMax (below, a sweep
+// warp per 2048 weights leaves most of the GPU idle: n = 10^6 has 489 of them
+// for 3648 resident warps), else kTile.
+inline bool fine_tiles(uint64_t n) { return n <= kFineMax; }
+inline uint32_t tile_count(uint64_t n)
+{
+    const uint64_t tile = fine_tiles(n) ? kFineTile : kTile;
+    return (uint32_t)((n + tile - 1) / tile);
+}
+// Most tiles, and list bytes, that a build of at most `cap` weights has.
+inline uint32_t tiles_cap(uint64_t cap)
+{
+    const uint32_t fine = tile_count(cap < kFineMax ? cap : kFineMax);
+    const uint32_t all = tile_count(cap);
+    return fine > all ? fine : all;
+}
+inline uint64_t slist_cap(uint64_t cap)
+{
+    const uint64_t fine = (uint64_t)tile_count(cap < kFineMax ? cap : kFineMax) * kSparseOf(kFineTile);
+    const uint64_t all = fine_tiles(cap) ? fine : (uint64_t)tile_count(cap) * kSparseOf(kTile);
+    return (fine > all ? fine : all) * sizeof(uint16_t);
+}
+
+struct Layout { // offsets in the workspace of a table of capacity cap
+    uint64_t hdr, part, agg, incl, cagg, cincl, flags, split, slist, total;
+};
+
+inline Layout layout_for(uint64_t cap)
+{
+    const uint32_t ntiles = tiles_cap(cap);
+    const uint32_t nchunks = (ntiles + kScanChunk - 1) / kScanChunk;
+    Layout L;
+    uint64_t o = 0;
+    L.hdr = o; o = align_up(o + sizeof(DevHeader), 256);
+    L.part = o; o = align_up(o + kMaxParts * sizeof(Partial), 256);
+    L.agg = o; o = align_up(o + (uint64_t)ntiles * sizeof(TileSum), 256);
+    L.incl = o; o = align_up(o + (uint64_t)ntiles * sizeof(TileSum), 256);
+    L.cagg = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
+    L.cincl = o; o = align_up(o + (uint64_t)nchunks * sizeof(TileSum), 256);
+    L.flags = o; o = align_up(o + (uint64_t)nchunks * sizeof(uint32_t), 256);
+    L.split = o; o = align_up(o + ((uint64_t)ntiles + 1) * sizeof(Split), 256);
+    L.slist = o; o = align_up(o + slist_cap(cap), 256);
+    L.total = o;
+    return L;
+}
+
+// Bytes of the buckets, before the workspace in the same allocation.
+inline uint64_t bucket_area(uint64_t cap) { return align_up(cap * sizeof(uint4), 256); }
+
 // ------------------------------------------------------------ 128-bit ops
 __device__ __forceinline__ u128 mk128(uint64_t lo, uint64_t hi) { return ((u128)hi << 64) | lo; }
 __device__ __forceinline__ uint64_t lo64(u128 v) { return (uint64_t)v; }

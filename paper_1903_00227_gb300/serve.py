@@ -41,7 +41,9 @@ from . import workloads as WL
 
 TABLE_MIN_CAP = 1 << 10
 BUCKET_BYTES = 16
-WORKSPACE_BYTES_PER_TILE = 2 * 48 + 16 + 64 + 16  # tile sums, split, member list, chunk share
+FINE_MAX = 1 << 22        # weights that a build cuts into tiles of 256; more take tiles of 2048
+TILE_BYTES = 3 * 48 + 1   # two tile sums, a split record, a share of a 256-tile chunk
+FIXED_BYTES = 68 << 10    # partial sums (64 KB), header, the records past the last tile, alignment
 
 
 def table_class(n: int) -> int:
@@ -50,9 +52,13 @@ def table_class(n: int) -> int:
 
 
 def table_bytes(cap: int) -> int:
-    """Device bytes of a table of capacity cap (buckets + workspace, rounded up)."""
-    tiles = (cap + 2047) // 2048
-    return cap * BUCKET_BYTES + tiles * WORKSPACE_BYTES_PER_TILE + (64 << 10)
+    """Device bytes of a table of capacity cap (buckets + workspace, rounded
+    up).  The workspace holds the tiles of any build up to cap: those of 256
+    of the first FINE_MAX weights (member lists of 16 B) or those of 2048 of
+    all of them (lists of 64 B)."""
+    fine = (min(cap, FINE_MAX) + 255) // 256
+    large = (cap + 2047) // 2048 if cap > FINE_MAX else 0
+    return cap * BUCKET_BYTES + max(fine, large) * TILE_BYTES + max(fine * 16, large * 64) + FIXED_BYTES
 
 
 @dataclasses.dataclass

@@ -229,3 +229,6 @@ extern "C" int sweep_host(const uint32_t *w, uint64_t n, int f32, uint32_t tile,
     *failed = hdr.pad[0];
     return g_stuck;
 }
+
+// Device bytes of a table of capacity cap: what wrs_table_create allocates.
+extern "C" uint64_t table_bytes_host(uint64_t cap) { return bucket_area(cap) + layout_for(cap).total; }

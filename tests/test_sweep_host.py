@@ -2,27 +2,20 @@
 warp (sweep_host.cpp): every bucket stored exactly once, none outside the
 table, and the table of Alg. 2, in every key mode, tile size and task length."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
 
 from oracle import wrs_oracle as O
 from paper_1903_00227_gb300 import workloads as WL
+from tests._host import host_library
 
-HERE = os.path.dirname(os.path.abspath(__file__))
-ROOT = os.path.dirname(HERE)
 U32_MAX = 0xFFFFFFFF
 
 
 @pytest.fixture(scope="module")
 def sweep(tmp_path_factory):
-    so = str(tmp_path_factory.mktemp("sweep") / "sweep_host.so")
-    subprocess.check_call(["g++", "-O1", "-w", "-std=gnu++17", "-DWRS_CHECK=1", "-shared", "-fPIC",
-                           "-I", os.path.join(ROOT, "paper_1903_00227_gb300", "csrc"), "-o", so,
-                           os.path.join(HERE, "sweep_host.cpp")])
-    f = ctypes.CDLL(so).sweep_host
+    f = host_library(tmp_path_factory.mktemp("sweep")).sweep_host
     f.argtypes = [ctypes.c_void_p, ctypes.c_uint64, ctypes.c_int, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int,
                   ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     f.restype = ctypes.c_int
