@@ -508,7 +508,7 @@ typedef struct {
     uint64_t q_lo, q_hi;  /* Q */
     uint64_t qp;          /* Q >> shift: the sampler's coin denominator */
     uint32_t light_max;   /* light iff raw word <= light_max */
-    uint32_t f32;         /* library: how the build reads the words */
+    uint32_t f32;         /* library: 1 if the weights were binary32 words */
     uint64_t n;
     uint64_t n_light;
     uint64_t reserved2[8]; /* [0], [1]: zero after a build of libwrs.so; the

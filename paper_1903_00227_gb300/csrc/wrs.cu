@@ -225,10 +225,10 @@ void launch_classify(uint32_t blocks, cudaStream_t s, bool f32, bool fine, const
 }
 
 void launch_split(cudaStream_t s, bool fine, const TileSum *incl, uint32_t ntiles, uint64_t n, DevHeader *hdr,
-                  Split *split)
+                  const Partial *part, Split *split)
 {
     auto *k = fine ? k_split<kFineTile> : k_split<kTile>;
-    k<<<ntiles / kThreads + 1, kThreads, 0, s>>>(incl, ntiles, n, hdr, split); // one boundary more than tiles
+    k<<<ntiles / kThreads + 1, kThreads, 0, s>>>(incl, ntiles, n, hdr, part, split); // one boundary more than tiles
 }
 
 void launch_sweep(cudaStream_t s, bool f32, bool fine, const uint32_t *w, uint64_t n, int vec, DevHeader *hdr,
@@ -287,7 +287,7 @@ wrs_status enqueue_build(wrs_table *t, const void *d_weights, uint64_t n, wrs_dt
         k_tilescan<<<nchunks, kThreads, 0, s>>>(t->hdr, t->agg, t->cagg, t->cincl, t->incl, t->flags, ntiles, epoch,
                                                 wait_limit, skip_tile);
         if (tm) cudaEventRecord(t->ev[4], s);
-        launch_split(s, fine, t->incl, ntiles, n, t->hdr, t->split);
+        launch_split(s, fine, t->incl, ntiles, n, t->hdr, t->part, t->split);
         if (o.acc == WRS_ACC_U64) k_require_u64<<<1, 32, 0, s>>>(t->hdr);
         if (tm) cudaEventRecord(t->ev[5], s);
         // a subproblem of the caller's split count (a run of tiles) is packed by one or more warps
@@ -804,7 +804,7 @@ extern "C" wrs_status wrs_build_noalloc(const void *d_weights, uint64_t n, wrs_d
     launch_classify(cls_blocks, s, f32, true, w, n, vec, hdr, agg, slist, ntiles);
     k_tilescan<<<nchunks, kThreads, 0, s>>>(hdr, agg, cagg, cincl, incl, flags, ntiles, kNaEpoch,
                                             g_wait_limit.load(), kNone);
-    launch_split(s, true, incl, ntiles, n, hdr, split);
+    launch_split(s, true, incl, ntiles, n, hdr, part, split);
     launch_sweep(s, f32, true, w, n, vec, hdr, split, slist, ntiles, buckets, sweep_group(ntiles, kSweepTiles), 0);
     return launch_err();
 }

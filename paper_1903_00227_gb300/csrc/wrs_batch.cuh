@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(kThreads) kb_stats(const uint32_t *__restrict_
 // One block per table; block 0 also advances the look-back generation.
 // Tables of at most kTile weights are built by kb_small instead.
 __global__ void __launch_bounds__(kThreads) kb_stats_combine(const BatchTable *__restrict__ bt,
-                                                             const Partial *__restrict__ part, uint32_t f32,
-                                                             DevHeader *hdr, uint32_t *epoch)
+                                                             Partial *part, uint32_t f32, DevHeader *hdr,
+                                                             uint32_t *epoch)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         uint32_t e = *epoch + 1;
@@ -102,7 +102,8 @@ __device__ __forceinline__ void small_build(const uint32_t *__restrict__ w, uint
     acc_fold(a, a64);
     a = acc_block_reduce(a);
     if (threadIdx.x == 0) {
-        s_status = write_header(a, N, F32, hdr);
+        uint32_t mode; // the sweep's: not needed
+        s_status = write_header(a, N, F32, hdr, mode);
         if (acc == WRS_ACC_U64 && s_status == 0 && hdr->q_hi != 0) s_status = hdr->status = kEOverflow;
     }
     __syncthreads();
@@ -178,12 +179,13 @@ template <int TILE>
 __global__ void __launch_bounds__(kThreads) kb_split(const BatchTable *__restrict__ bt,
                                                      const BlockMap *__restrict__ map,
                                                      const TileSum *__restrict__ incl, DevHeader *hdr,
-                                                     Split *__restrict__ split)
+                                                     const Partial *__restrict__ part, Split *__restrict__ split)
 {
     const BlockMap m = map[blockIdx.x];
     const BatchTable &T = bt[m.table];
-    split_body<TILE>(incl + T.tile0, T.ntiles, T.n, hdr + m.table, split + T.tile0 + m.table, // one boundary more than tiles
-               m.local * kThreads + threadIdx.x);
+    split_body<TILE>(incl + T.tile0, T.ntiles, T.n, hdr + m.table, part + T.part0,
+                     split + T.tile0 + m.table, // one boundary more than tiles
+                     m.local * kThreads + threadIdx.x);
 }
 
 template <int F32, int TILE>
@@ -390,7 +392,7 @@ wrs_status batch_enqueue_build(wrs_batch *b, const uint32_t *w, uint32_t f32, cu
     kb_tilescan<<<b->nb[kMapScan], kThreads, 0, s>>>(b->d_tables, b->map[kMapScan], b->hdr, b->agg, b->cagg,
                                                       b->cincl, b->incl, b->flags, b->epoch, g_wait_limit.load());
     auto *split = b->fine ? kb_split<kFineTile> : kb_split<kTile>;
-    split<<<b->nb[kMapSplit], kThreads, 0, s>>>(b->d_tables, b->map[kMapSplit], b->incl, b->hdr, b->split);
+    split<<<b->nb[kMapSplit], kThreads, 0, s>>>(b->d_tables, b->map[kMapSplit], b->incl, b->hdr, b->part, b->split);
     if (sweep0) cudaEventRecord(sweep0, s);
     batch_launch_sweep(b, w, vec, f32, s);
     if (sweep1) cudaEventRecord(sweep1, s);

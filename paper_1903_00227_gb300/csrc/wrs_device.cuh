@@ -40,9 +40,9 @@ struct DevHeader {
     uint64_t q_lo, q_hi;    // Q
     uint64_t qp;            // Q >> shift
     uint32_t light_max;     // light iff raw word <= light_max
-    uint32_t f32;           // bit 0: binary32 weights; bits 8 and up: the sweep's PackMode
+    uint32_t f32;           // 1: binary32 weights
     uint64_t n;
-    uint64_t n_light;       // filled by the sweep of the last tile
+    uint64_t n_light;       // written after the light count: by k_split, k_small or k_pp_local
     uint64_t pad[2];        // zero; the check build counts failed checks in pad[0]
 };
 
@@ -50,7 +50,8 @@ struct Partial {            // per-block result of k_stats
     uint64_t lo, hi;        // exact partial sum (units of 2^base)
     int32_t base;           // INT_MAX: no nonzero weight seen
     uint32_t flags;         // bit 0 invalid weight, bit 1 range exceeded
-    uint32_t mx, pad;       // largest word
+    uint32_t mx;            // largest word
+    uint32_t mode;          // first partial, from k_stats_combine on: the sweep's PackMode
 };
 constexpr uint32_t kPartInvalid = 1u, kPartOverflow = 2u;
 
@@ -67,7 +68,7 @@ struct Split {              // result of k_split per tile boundary (48 B; ntiles
     uint32_t hb;            // tile holding the heavy current at the first light from this tile on
     uint32_t next_heavy;    // position of the first heavy item after this tile
     uint32_t nheavy;        // heavy items in this tile
-    uint32_t ch;            // heavy items before this tile
+    uint32_t mode;          // the sweep's PackMode, the same in every record
     uint64_t d_lo, d_hi;    // D of the first light from this tile on
     uint64_t e_lo, e_hi;    // E after the heavies before this tile
 };

@@ -287,7 +287,7 @@ __device__ __forceinline__ void stats_body(const uint32_t *__restrict__ w, uint6
     a = acc_block_reduce(a);
     if (threadIdx.x == 0) {
         Partial p;
-        p.lo = lo64(a.acc); p.hi = hi64(a.acc); p.base = a.base; p.flags = a.flags; p.mx = a.mx; p.pad = 0;
+        p.lo = lo64(a.acc); p.hi = hi64(a.acc); p.base = a.base; p.flags = a.flags; p.mx = a.mx; p.mode = 0;
         *out = p;
     }
 }
@@ -316,9 +316,9 @@ __device__ bool f32_light(uint32_t v, uint64_t n, u128 Q, int beta)
     return nm <= (Q << dd);
 }
 
-__device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint32_t f32, DevHeader *hdr);
+__device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint32_t f32, DevHeader *hdr, uint32_t &mode);
 
-__device__ __forceinline__ void stats_combine_body(const Partial *__restrict__ part, uint32_t nparts, uint64_t n,
+__device__ __forceinline__ void stats_combine_body(Partial *part, uint32_t nparts, uint64_t n,
                                                    uint32_t f32, DevHeader *hdr)
 {
     Acc a;
@@ -331,12 +331,14 @@ __device__ __forceinline__ void stats_combine_body(const Partial *__restrict__ p
         acc_merge(a, b);
     }
     a = acc_block_reduce(a);
-    if (threadIdx.x == 0) write_header(a, n, f32, hdr);
+    // every thread has read its partials before the reduction's barrier
+    if (threadIdx.x == 0) write_header(a, n, f32, hdr, part[0].mode);
 }
 
 // The table header from the exact total (thread 0): status, beta, Q, shift,
-// qp and the light threshold on the raw words.
-__device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint32_t f32, DevHeader *hdr)
+// qp and the light threshold on the raw words; and how the sweep forms n q and
+// its keys (PackMode), which is not the caller's business and goes to `mode`.
+__device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint32_t f32, DevHeader *hdr, uint32_t &mode)
 {
     uint32_t status = kOk;
     if (a.flags & kPartInvalid) status = kEInval;
@@ -366,14 +368,13 @@ __device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint3
     hdr->q_hi = hi64(Q);
     hdr->qp = lo64(Q >> shift);
     hdr->light_max = light_max;
-    // how the sweep forms n q and its keys (PackMode)
-    uint32_t mode = kPackQ128;
+    mode = kPackQ128;
     if (shift == 0 && bitlen128(Q) + (32 - __clz((int)(uint32_t)n)) <= 95) {
         const bool normal = !f32 || beta >= -94;
         if (normal && (!f32 || (int)(a.mx >> 23) <= 158 + beta)) mode = kPackQ32;
         else if (normal && (int)(light_max >> 23) <= 158 + beta) mode = kPackQ96;
     }
-    hdr->f32 = f32 | mode << 8;
+    hdr->f32 = f32;
     hdr->n = n;
     hdr->n_light = 0;
     hdr->pad[0] = 0;
@@ -383,7 +384,7 @@ __device__ __forceinline__ uint32_t write_header(const Acc &a, uint64_t n, uint3
     return status;
 }
 
-__global__ void __launch_bounds__(kThreads) k_stats_combine(const Partial *__restrict__ part, uint32_t nparts,
+__global__ void __launch_bounds__(kThreads) k_stats_combine(Partial *part, uint32_t nparts,
                                                             uint64_t n, uint32_t f32, DevHeader *hdr)
 {
     stats_combine_body(part, nparts, n, f32, hdr);
@@ -732,8 +733,7 @@ __global__ void __launch_bounds__(kThreads) k_tilescan(DevHeader *hdr, const Til
 // ------------------------------------------------------------ k_split
 // For every tile boundary c = 0 .. ntiles, from the tile prefix sums: the
 // keys there (D: of the first light from tile c on, E: after the heavies
-// before tile c), the rank of the first heavy from tile c on, the tile's
-// heavies, and
+// before tile c), the tile's heavies, the table's PackMode, and
 //   hb = max{ b : E(b) <= D(c) }  -- the tile holding the first heavy item
 //        with E > D(c), the heavy current when the first light from tile c
 //        on is packed (the split of Alg. 3 on the heavy prefix sums);
@@ -759,10 +759,11 @@ template <int TILE> __device__ __forceinline__ Prefix prefix_at(const TileSum *i
 __device__ __forceinline__ u128 key_E(const Prefix &p, uint64_t n, u128 Q) { return times_n(p.H, n) - (u128)p.ch * Q; }
 __device__ __forceinline__ u128 key_D(const Prefix &p, uint64_t n, u128 Q) { return (u128)p.cl * Q - times_n(p.L, n); }
 
-// Boundary c of one table (one thread per boundary).
+// Boundary c of one table (one thread per boundary); part: its first partial.
 template <int TILE>
 __device__ __forceinline__ void split_body(const TileSum *__restrict__ incl, uint32_t ntiles, uint64_t n,
-                                           DevHeader *hdr, Split *__restrict__ split, uint32_t c)
+                                           DevHeader *hdr, const Partial *__restrict__ part,
+                                           Split *__restrict__ split, uint32_t c)
 {
     if (*(volatile uint32_t *)&hdr->status) return;
     const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
@@ -780,7 +781,7 @@ __device__ __forceinline__ void split_body(const TileSum *__restrict__ incl, uin
     s.hb = lo;
     s.nheavy = 0;
     s.next_heavy = kNone;
-    s.ch = (uint32_t)pc.ch;
+    s.mode = part->mode;
     s.d_lo = lo64(Dc); s.d_hi = hi64(Dc);
     s.e_lo = lo64(Ec); s.e_hi = hi64(Ec);
     if (c < ntiles) {
@@ -804,9 +805,10 @@ __device__ __forceinline__ void split_body(const TileSum *__restrict__ incl, uin
 
 template <int TILE>
 __global__ void __launch_bounds__(kThreads) k_split(const TileSum *__restrict__ incl, uint32_t ntiles, uint64_t n,
-                                                    DevHeader *hdr, Split *__restrict__ split)
+                                                    DevHeader *hdr, const Partial *__restrict__ part,
+                                                    Split *__restrict__ split)
 {
-    split_body<TILE>(incl, ntiles, n, hdr, split, blockIdx.x * kThreads + threadIdx.x);
+    split_body<TILE>(incl, ntiles, n, hdr, part, split, blockIdx.x * kThreads + threadIdx.x);
 }
 
 // ------------------------------------------------------------ k_sweep
@@ -1202,7 +1204,7 @@ __device__ __forceinline__ void sweep_body(const uint32_t *__restrict__ w, uint6
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (__shfl_sync(0xFFFFFFFFu, *(volatile const uint32_t *)&hdr->status, 0)) return; // the whole warp or none
     const u128 Q = mk128(hdr->q_lo, hdr->q_hi);
-    const uint32_t mode = force_wide ? (uint32_t)kPackQ128 : hdr->f32 >> 8; // the same for the whole grid
+    const uint32_t mode = force_wide ? (uint32_t)kPackQ128 : split_head(split + c_first).w; // the table's
     bool bad;
     if (mode == kPackQ32)
         bad = sweep_task<F32, kPackQ32, TILE>(*reinterpret_cast<WarpRings<kPackQ32> *>(smem_raw), w, n, vec, hdr, split,

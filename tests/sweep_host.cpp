@@ -174,7 +174,8 @@ void build(const uint32_t *w, uint64_t n, int vec, uint32_t group, bool wide, De
         acc_take<F32>(a, a64, w[i]);
         acc_fold(a, a64);
     }
-    if (write_header(a, n, F32, hdr)) return;
+    Partial part;
+    if (write_header(a, n, F32, hdr, part.mode)) return;
     const uint32_t ntiles = (uint32_t)((n + TILE - 1) / TILE);
     std::vector<TileSum> incl(ntiles);
     std::vector<Split> split(ntiles + 1);
@@ -198,7 +199,7 @@ void build(const uint32_t *w, uint64_t n, int vec, uint32_t group, bool wide, De
         s.cl = cl;
         s.l_lo = lo64(L); s.l_hi = hi64(L); s.h_lo = lo64(H); s.h_hi = hi64(H);
     }
-    for (uint32_t c = 0; c <= ntiles; ++c) split_body<TILE>(incl.data(), ntiles, n, hdr, split.data(), c);
+    for (uint32_t c = 0; c <= ntiles; ++c) split_body<TILE>(incl.data(), ntiles, n, hdr, &part, split.data(), c);
     for (uint32_t c = 0; c < ntiles; c += group) {
         memset(smem_raw, 0xA5, sizeof(smem_raw));
         run_warp([&] {
