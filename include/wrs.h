@@ -343,15 +343,15 @@ wrs_status wrs_batch_download(const wrs_batch *b, void *h_buckets, uint64_t byte
  * number of split subproblems of a table is its tiles / group; a batch of at
  * most 2^22 weights in all is cut into tiles of 256).  wrs_batch_tune builds
  * the batch from d_weights, then for each class present times the sweep
- * with group 1, 2, 4 and 8 (best of three each, CUDA events) and keeps the
+ * with group 1, 2 and 4 (best of three each, CUDA events) and keeps the
  * fastest; finally it rebuilds with the chosen groups and writes the tuned
  * sweep time to *h_sweep_ms when not NULL.  Synchronous.  The groups change
  * speed only, never a bucket. */
 #define WRS_BATCH_CLASSES 5
 wrs_status wrs_batch_tune(wrs_batch *b, const void *d_weights, wrs_dtype dtype, void *stream,
                           float *h_sweep_ms);
-wrs_status wrs_batch_groups(const wrs_batch *b, uint32_t *h_groups);             /* WRS_BATCH_CLASSES entries */
-wrs_status wrs_batch_set_groups(wrs_batch *b, const uint32_t *h_groups);         /* each 1..64; synchronous */
+wrs_status wrs_batch_groups(const wrs_batch *b, uint32_t *h_groups);             /* WRS_BATCH_CLASSES entries, as set */
+wrs_status wrs_batch_set_groups(wrs_batch *b, const uint32_t *h_groups);         /* each 1..64 (above 4 runs as 4); synchronous */
 
 /* Free all memory of the batch (synchronises the device first).  NULL ok. */
 void wrs_batch_free(wrs_batch *b);

@@ -36,7 +36,8 @@ struct BlockMap {         // one per block of a batch launch
 };
 
 constexpr int kBatchClasses = WRS_BATCH_CLASSES; // sweep size classes by tiles: 1, 2-4, 5-32, 33-256, more
-constexpr uint32_t kBatchGroups[] = {1, 2, 4, 8}; // tuner's candidates for own tiles per sweep warp
+constexpr uint32_t kBatchGroups[] = {1, 2, 4}; // tuner's candidates for own tiles per sweep warp
+static_assert(kBatchGroups[2] <= (uint32_t)kSweepTiles, "apply_groups runs larger groups as kSweepTiles");
 constexpr uint32_t kBatchPartWeights = 16384;    // weights per k_stats block (at least)
 
 inline int batch_class(uint64_t n)
