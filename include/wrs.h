@@ -239,8 +239,8 @@ const char *wrs_status_str(wrs_status s);
  *     build that wrote each bucket exactly once (Alg. 2 and Alg. 3 assign
  *     every bucket to one step) leaves 1 in every reserved word, and a
  *     missed or doubled bucket shows as 0 or 2 in the downloaded table;
- *   - a bucket index or alias outside the table, a shared-memory index of
- *     the sweep outside its window, a sweep subproblem that ends in another
+ *   - a bucket index or alias outside the table, a ring of the sweep in
+ *     shared memory over its capacity, a sweep subproblem that ends in another
  *     heavy tile than the split search gave the next one (Alg. 3: the state
  *     at the end of one subproblem is the start of the next), and a sampled
  *     bucket whose alias lies outside the table each count as a failed

@@ -224,9 +224,8 @@ __device__ __forceinline__ void set_status(DevHeader *h, uint32_t code)
 // bucket store adds one to the bucket's reserved fourth word instead of
 // storing 0 (the build clears the buckets first, so a table in which every
 // bucket was written exactly once has 1 in every reserved word), a bucket
-// index or alias outside the table is refused, and the index checks placed
-// on the sweep's shared-memory reads and on its end-of-subproblem state
-// hold.  A check that fails counts itself in the header's first reserved
+// index or alias outside the table is refused, and the fill of the sweep's
+// rings and its end-of-subproblem state are checked.  A check that fails counts itself in the header's first reserved
 // word, sets WRS_EINTERNAL and skips the access.  In the standard build all
 // of this compiles away and the reserved word is stored as 0.
 #ifndef WRS_CHECK

@@ -902,6 +902,7 @@ __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *_
     if (lane == 0) R.put(R.light(0), drun, 0u, kNone);
 
     for (;;) {
+        check_ok(lh - li < kRing && hh - hj < kRing, hdr); // the rings hold their entries and the end entry
         if (lh - li < 32 && at < end && (hh != hj || s >= ntiles)) { // the next own weights
             // Direct: the current heavy reaches past every light of the next
             // batches, so these lights go straight from the weights to their buckets.
