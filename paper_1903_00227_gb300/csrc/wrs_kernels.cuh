@@ -851,6 +851,7 @@ constexpr uint32_t kDirect = 128;        // weights a warp packs at once under o
 // 3.61 / 3.81 ms for n = 10^9 Zipf 1.5, and 6.98 / 6.63 / 6.54 / 6.57 / - ms
 // for n = 6*10^8 Zipf 0.8.  (The 32-bit keys would cover 2^14 Q, eight tiles.)
 constexpr int kSweepTiles = 4;
+static_assert(kSweepTiles * kTile <= 1 << kTaskBits, "the 32-bit keys' range");
 
 template <int F32, int MODE, int TILE>
 __device__ __forceinline__ bool sweep_task(WarpRings<MODE> &R, const uint32_t *__restrict__ w, uint64_t n, int vec,

@@ -1,6 +1,7 @@
 // wrs_pack.cuh -- the packing core of the sweep: Alg. 2 run by one warp on a
 // stream of light and a stream of heavy items.  Included by wrs_kernels.cuh
-// only.
+// only.  Where a function is written in PTX, a second form without it lets
+// the host compiler build the sweep, whose tests check every bucket store.
 //
 // With the keys of wrs_kernels.cuh (D[i]: deficits of the lights before
 // light i; E[j]: excesses of the heavies up to and including heavy j) Alg. 2
@@ -91,11 +92,6 @@ __device__ __forceinline__ K128 kmul(K128 a, uint32_t c)
     return r;
 }
 template <typename K> __device__ __forceinline__ bool kle(K a, K b) { return !kneg(ksub(b, a)); } // |b - a| in range
-__device__ __forceinline__ uint4 kpack(K96 a) { return make_uint4((uint32_t)a.lo, (uint32_t)(a.lo >> 32), a.hi, 0u); }
-__device__ __forceinline__ uint4 kpack(K128 a)
-{
-    return make_uint4((uint32_t)a.lo, (uint32_t)(a.lo >> 32), (uint32_t)a.hi, (uint32_t)(a.hi >> 32));
-}
 template <typename K> __device__ __forceinline__ K kunpack(uint4 v);
 template <> __device__ __forceinline__ K96 kunpack<K96>(uint4 v)
 {
@@ -263,7 +259,8 @@ template <int MODE> struct WarpRings {
     static constexpr bool kWide = MODE == kPackQ128;
     static constexpr int kPer = kWide ? 2 : 4;             // weights a lane reads at once
     static constexpr uint32_t kBatch = 32 * kPer;
-    static constexpr uint32_t kRing = kWide ? 128 : 256;   // entries of a ring: 32 left over, a batch and an end entry fit
+    static constexpr uint32_t kRing = kWide ? 128 : 256;   // entries of a ring
+    static_assert(32 + kBatch + 1 <= kRing, "what is left over, a batch and an end entry");
     uint64_t low[2 * kRing];
     uint2 kp[2 * kRing];     // (32-bit key, position)
     uint32_t high[kWide ? 2 * kRing : 1];
@@ -281,7 +278,12 @@ static_assert(sizeof(WarpRings<kPackQ128>) <= kPackSmemBytes, "rings");
 
 // 32-bit keys: the relative key shifted down so that every D of the task is
 // below 2^30.  Equal ones are told apart by the exact low words (they differ
-// by less than 2^63, or 2^95 in the wide mode).
+// by less than 2^63, or 2^95 in the wide mode).  A task has at most 2^kTaskBits
+// lights, so its D span less than 2^(64 + kTaskBits), as Q < 2^64, or
+// 2^(kQBits + kTaskBits) in the wide mode, and 30 bits of that stay above the shift.
+constexpr int kTaskBits = 13;
+static_assert(64 + kTaskBits - 30 < 63, "kshr32 of a K96, and ties in 64 bits");
+static_assert(kQBits + kTaskBits - 30 < 95, "kshr32 of a K128, and ties in 96 bits");
 template <typename K> struct KeyFrame {
     K dmax;        // last D of the task, relative to its first
     uint32_t s;
