@@ -109,16 +109,16 @@ wrs_status wrs_table_build(wrs_table *t, const void *d_weights, uint64_t n,
  * is cut and which exact arithmetic the pack uses.
  *   splits  number of subproblems of Alg. 3's pack, each a run of
  *           consecutive 2048-weight tiles; 0: the library's choice; at most
- *           the number of tiles, ceil(n / 2048).  A run is packed by one warp
- *           of the sweep, or by several where the runs are longer than four
- *           tiles or too few to fill the GPU
+ *           the number of tiles, ceil(n / 2048).  An upper bound for the
+ *           length of the runs only: a warp of the sweep packs at most four
+ *           tiles, fewer where that leaves the GPU idle
  *   tile    0 or 2048 (fixed)
  *   window  0 or 2048 (fixed)
  *   acc     WRS_ACC_AUTO: 64-bit bucket arithmetic when Q < 2^64, else
  *           128-bit; WRS_ACC_U64: the build fails with WRS_EOVERFLOW (in
  *           the status word) when Q >= 2^64; WRS_ACC_U128: 128-bit
- *           arithmetic throughout.  Keys are 128-bit in every mode.  There
- *           is no binary64 mode: every mode is exact.
+ *           arithmetic throughout.  Keys are exact in every mode (96 bits
+ *           where n Q < 2^95, else 128).  There is no binary64 mode.
  *   flags   0 */
 typedef enum { WRS_ACC_AUTO = 0, WRS_ACC_U64 = 1, WRS_ACC_U128 = 2 } wrs_acc;
 typedef struct {
