@@ -828,7 +828,11 @@ __global__ void __launch_bounds__(kThreads) k_split(const TileSum *__restrict__ 
 // weight at 70 % issue; about 290 per batch of own weights, 320 per batch of
 // heavies' tile, 115 per search and 64 per 32 buckets stored).  It replaces a
 // block per eight tiles with 128-bit keys of a whole tile in shared memory, a
-// merge walked by threads and five barriers a tile.  n = 10^8, uniform / Zipf
+// merge walked by threads and five barriers a tile.  It moves 41 B of DRAM per
+// weight for 20 of work (uniform): outputs leave in merge order, where a light's
+// and a heavy's 16-byte buckets share 32-byte sectors, and the resident warps'
+// tasks span some 480 MB of buckets, so the L2 evicts sectors half written.
+// n = 10^8, uniform / Zipf
 // 0.8 / Zipf 1.5: 1.54 / 1.50 / 1.18 -> 1.18 / 1.22 / 0.42 ms; n = 10^9 uniform
 // 15.4 -> 10.9 ms, Zipf 1.5 12.2 -> 3.6 ms.  One warp per block: the scheduler
 // replaces each warp as it ends, 19 -> 23 resident warps per SM (1.47 -> 1.40 ms

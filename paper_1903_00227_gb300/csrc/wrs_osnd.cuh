@@ -303,7 +303,7 @@ __device__ __forceinline__ void os_push(uint32_t level, uint32_t member, uint64_
 }
 
 // One frontier entry per block iteration.  SRC as k2_group.  Bound by binary64
-// throughput (76 % of its pipe): n = 10^6 Zipf 1.0, k = 10^8 2.61 ms when each
+// throughput (79 % of its pipe): n = 10^6 Zipf 1.0, k = 10^8 2.61 ms when each
 // thread finished its node's deviate on its own, 2.14 ms in two passes, 1.6 ms
 // with the second one's kinds apart.  Where a group's samples fall on few of
 // its items, by the latency of a depth: three blocks per SM, as many as the

@@ -11,9 +11,10 @@
 // the heavies before light l among the next 32 by a five-step shuffle search,
 // one OR-reduction gives the merged order, and lane p writes the buckets of the
 // p-th and the (32 + p)-th item.  So a step costs the same whatever the mix of lights and
-// heavies, no lane idles, a warp's stores go to near positions (16-byte
-// stores by lanes that each own a run of items cost 6.7 to 10 ms per 10^9
-// buckets on a GB300, consecutive ones 2.1 ms), and no warp waits for another.
+// heavies, no lane idles, a warp's stores go to two runs of near positions, the
+// lights' and the heavies' (16-byte stores by lanes that each own a run of items
+// cost 6.7 to 10 ms per 10^9 buckets on a GB300, consecutive ones 2.1 ms), and no
+// warp waits for another.
 #pragma once
 
 namespace wrs {

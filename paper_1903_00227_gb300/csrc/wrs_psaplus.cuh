@@ -247,8 +247,10 @@ __device__ __forceinline__ bool pp_tile(GroupSmem &S, const uint32_t (&x)[kItems
 }
 
 // One tile per block.  64-bit keys when every n q of the tile and Q lie below
-// 2^51, so that its sums stay below 2^62 (n = 10^8 uniform weights do); other
-// tiles take 128 bits.  Bound by instruction issue: n = 10^8 uniform 1.40 ms
+// 2^51, so that its sums stay below 2^62: 24-bit uniform weights do up to n of
+// about 1.3 10^8; at n = 10^9 n q has 54 bits and every tile takes 128 (the
+// whole build 18.1 -> 17.3 ms only).  Bound by shared-memory wavefronts and
+// issue (L1 data pipe 70 % busy, issue 63 %, ALU 61 %): n = 10^8 uniform 1.40 ms
 // with 128-bit keys only (11.4 warp instructions per weight), 1.12 ms with
 // 64-bit keys (8.4), 1.00 ms with the keys written once (own_keys); the whole
 // build 1.41 -> 1.35 ms with the header read beside the weights (Zipf 1.5, on

@@ -141,9 +141,10 @@ template <> __device__ __forceinline__ uint64_t thr_of<uint64_t>(uint64_t bw, ui
 // written once, from registers, instead of by an in-place prefix over stored
 // deficits (two more passes through shared memory).  With the members' q in 64
 // bits and one scan of the warps' totals: k2_group, Zipf 0.8 at n = 10^8, 0.98
-// -> 0.81 ms.  Bound by instruction issue (8.4 warp instructions per weight at
-// 68 % before); staging the buckets so that they are stored in item order was
-// no faster (1.00 ms).
+// -> 0.81 ms.  Bound by shared-memory wavefronts, most of them from the
+// threads' searches and walks at scattered rows (uniform, n = 10^8: L1 data pipe
+// 82 % busy, ALU 71 %, issue 67 %); staging the buckets so that they are stored
+// in item order was no faster (1.00 ms).
 template <typename K>
 struct OwnKeys {
     uint32_t nl, nh;      // lights and heavies of the block
